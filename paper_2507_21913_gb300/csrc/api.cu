@@ -209,7 +209,7 @@ static void free_plan(hpfmm_plan *pl) {
                   pl->ab_key, pl->ab_lo, pl->ab_hi, pl->ab_parent, pl->ab_lvl, pl->ab_child,
                   pl->ab_cut, pl->ab_off, pl->ab_idx, pl->ab_lev, pl->ab_btot, pl->ab_lrank,
                   pl->ab_leaf, pl->near, pl->loclo, pl->dgeom, pl->tree_ctr, pl->ctr, pl->mir_A, pl->mir_B,
-                  pl->tree_tmp, pl->in_xy};
+                  pl->tree_tmp, pl->in_xy, pl->fxy, pl->fq, pl->near64, pl->qexp};
   for (void *b : bufs)
     if (b) cudaFree(b);
   delete pl;
@@ -461,9 +461,15 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
   if (f32) ALLOC(pl->yabs, sizeof(float) * n);
   if (f32) ALLOC(pl->loclo, sizeof(float2) * n);
   if (f32 && !pl->adaptive) ALLOC(pl->near, sizeof(float4) * n);
-  if (f32 && !pl->adaptive) {  // mirror M2L results: rows 0 and 1 of levels 1..H
-    ALLOC(pl->mir_A, sizeof(cf) * 4 * (((size_t)1 << pl->H) - 1) * P1);
-    ALLOC(pl->mir_B, sizeof(cf) * 4 * (((size_t)1 << pl->H) - 1) * P1);
+  if (!pl->adaptive) {  // mirror M2L results: rows 0 and 1 of levels 1..H
+    ALLOC(pl->mir_A, csz * 4 * (((size_t)1 << pl->H) - 1) * P1);
+    ALLOC(pl->mir_B, csz * 4 * (((size_t)1 << pl->H) - 1) * P1);
+  }
+  if (!f32) {
+    ALLOC(pl->fxy, sizeof(longlong2) * n);
+    ALLOC(pl->fq, sizeof(float2) * n);
+    ALLOC(pl->near64, 3 * sizeof(double) * n);
+    ALLOC(pl->qexp, sizeof(int));
   }
   ALLOC(pl->t_m2m, tf * 4 * m2);
   ALLOC(pl->t_l2l, tf * 4 * m2);
@@ -494,6 +500,7 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
   s = fmm_set_smem_limits(p);
   if (s == HPFMM_OK) s = fmm_prepare();
   if (s == HPFMM_OK) s = adaptive_prepare();
+  if (s == HPFMM_OK) s = near64_prepare();
   if (s != HPFMM_OK) { free_plan(pl); return s; }
   {
     // the far-field streams of a split evaluation -- side (S2M, M2M, coarse
@@ -534,6 +541,7 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
   cudaError_t e = cudaMemsetAsync(pl->status, 0, sizeof(int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->tree_ctr, 0, sizeof(unsigned), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->ctr, 0, kCtrSlots * sizeof(int), st);
+  if (e == cudaSuccess && pl->qexp) e = cudaMemsetAsync(pl->qexp, 0, sizeof(int), st);
   if (e != cudaSuccess) {
     set_last_error("hpfmm_create: %s", cudaGetErrorString(e));
     free_plan(pl);

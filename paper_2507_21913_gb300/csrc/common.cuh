@@ -410,6 +410,12 @@ struct hpfmm_plan {
   cudaEvent_t ev_up = nullptr;
   void *mir_A = nullptr, *mir_B = nullptr;
   float4 *near = nullptr;  // near-field sums per point (sorted order)
+  // double-precision plans (near64.cu): fixed-point coordinates and split
+  // charges of the free-space pairs, the sums (3 n doubles), the biased
+  // exponent of the largest charge (zeroed by the evaluation's last kernel)
+  void *fxy = nullptr, *fq = nullptr;
+  double *near64 = nullptr;
+  int *qexp = nullptr;
   double *hgeo = nullptr;  // pinned host copy of geo, written by the tree build
   int *status = nullptr;  // device status word
   double *geo = nullptr;  // device: x0, side, invalid flag, 2^30/side, largest leaf (int)
@@ -481,6 +487,13 @@ hpfmm_status adaptive_alloc(hpfmm_plan *pl);
 // device (a synchronous copy, so done at plan creation and never inside a
 // stream capture such as the batched graph)
 hpfmm_status fmm_prepare();
+hpfmm_status near64_prepare();
+// near field of a double-precision plan (near64.cu): the free-space pair sums
+// to pl->near64, the bottom row's image and reaction pairs to the outputs
+hpfmm_status near64_launch(hpfmm_plan *pl, const double *qs, cudaStream_t st);
+int near64_kernels(const hpfmm_plan *pl);  // kernels it launches
+hpfmm_status mirror64_launch(hpfmm_plan *pl, const double *qs, double *pot, double *grad,
+                             cudaStream_t st);
 hpfmm_status adaptive_prepare();
 hpfmm_status fmm_eval_targets(hpfmm_plan *pl, const double *q, const double *xt,
                               const double *yt, int64_t nt, const int64_t *blist,

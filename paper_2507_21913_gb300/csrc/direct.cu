@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(kDirectThreads)
 direct_kernel(const double *__restrict__ xs, const double *__restrict__ ys,
               const double *__restrict__ qs, int64_t ns, const double *__restrict__ xt,
               const double *__restrict__ yt, const int64_t *__restrict__ self_index,
-              int64_t nt, cd kappa, double *__restrict__ pot, double *__restrict__ grad,
+              int64_t nt, KappaLog K, double *__restrict__ pot, double *__restrict__ grad,
               int64_t chunk, double *__restrict__ part) {
   __shared__ double sx[kDirectThreads], sy[kDirectThreads], sq[kDirectThreads];
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -44,8 +44,7 @@ direct_kernel(const double *__restrict__ xs, const double *__restrict__ ys,
       double q = sq[k];
       if (base + k != self) pair_free(acc, dx, y - sy[k], q);
       double Y = y + sy[k];
-      pair_image(acc, dx, Y, q);
-      pair_reaction_d(acc, dx, Y, q, kappa);
+      pair_mirror_d(acc, dx, Y, q, K);
     }
   }
   if (!active) return;
@@ -110,10 +109,11 @@ extern "C" hpfmm_status hpfmm_direct(const double *xs, const double *ys, const d
   cudaStream_t st = (cudaStream_t)stream;
   HP_TRY(special_init_here());
   int64_t blocks = (nt + kDirectThreads - 1) / kDirectThreads;
-  // few targets: split the sources over a second grid dimension (at least
-  // 4 blocks per SM in all, at least 2048 sources per chunk)
-  int64_t nchunk = (4 * 152 + blocks - 1) / blocks;
-  const int64_t maxc = (ns + 2047) / 2048;
+  // few targets: split the sources over a second grid dimension (about 8
+  // blocks per SM in all, at least 512 sources per chunk: 256 targets of 200003
+  // sources took 308 ms with 196 blocks and the earlier pair, 38 ms now)
+  int64_t nchunk = (8 * 152 + blocks - 1) / blocks;
+  const int64_t maxc = (ns + 511) / 512;
   if (nchunk > maxc) nchunk = maxc;
   if (nchunk < 1) nchunk = 1;
   if (nchunk > 65535) nchunk = 65535;
@@ -121,7 +121,7 @@ extern "C" hpfmm_status hpfmm_direct(const double *xs, const double *ys, const d
   double *part = nullptr;
   if (nchunk > 1) HP_CUDA(cudaMallocAsync((void **)&part, sizeof(double) * 6 * nchunk * nt, st));
   direct_kernel<<<dim3((unsigned)blocks, (unsigned)nchunk), kDirectThreads, 0, st>>>(
-      xs, ys, qs, ns, xt, yt, self_index, nt, mk(kappa_re, kappa_im), pot, grad, chunk, part);
+      xs, ys, qs, ns, xt, yt, self_index, nt, kappa_log(kappa_re, kappa_im), pot, grad, chunk, part);
   if (part) {
     direct_reduce<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(part, (int)nchunk, nt, pot, grad);
     cudaFreeAsync(part, st);

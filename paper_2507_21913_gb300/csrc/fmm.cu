@@ -50,13 +50,31 @@ constexpr int kWarpsPerBlock = 4;
 // --------------------------------------------------------------------------
 // gather the charges into tree order
 // (blockIdx.y = RHS; qsm, when given, also receives the charges point-major:
-// qsm[k * rp + r], for the multi-RHS near field)
+// qsm[k * rp + r], for the multi-RHS near field; qexp, when given, the biased
+// exponent of the largest charge, for the double-precision near field's split)
 template <typename R>
-__global__ void k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm,
-                           int64_t n, R *__restrict__ qs, R *__restrict__ qsm, int rp) {
+__global__ void __launch_bounds__(256)
+k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm,
+                           int64_t n, R *__restrict__ qs, R *__restrict__ qsm, int rp,
+                           int *__restrict__ qexp) {
   pdl_wait();  // launched as a dependent of the tree build's last kernel
   pdl_trigger();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if constexpr (sizeof(R) == 8) {
+    if (qexp) {
+      __shared__ int smax;
+      if (threadIdx.x == 0) smax = 0;
+      __syncthreads();
+      const double v = k < n ? q[perm[k]] : 0.0;
+      if (k < n) qs[k] = v;
+      const int e = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
+      const int m = __reduce_max_sync(0xffffffffu, e);
+      if ((threadIdx.x & 31) == 0) atomicMax(&smax, m);
+      __syncthreads();
+      if (threadIdx.x == 0 && smax > 0) atomicMax(qexp, smax);
+      return;
+    }
+  }
   if (k >= n) return;
   const int r = blockIdx.y;
   const double qd = q[(size_t)r * n + perm[k]];
@@ -446,12 +464,15 @@ k_m2m_level(int l, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restrict__ 
 // instead of launches for the coarse levels.  It then pushes the expansions
 // down the subtree in shared memory (child = L2L(parent) + the child's own M2L
 // result).  Without EVAL the leaf expansions are written to global memory;
-// with EVAL (single-precision split evaluation) they stay in shared memory and
-// the block evaluates them at its points (L2P, Eq. truncatedLE), adds the
-// near-field sums of k_near32 and writes the outputs.
+// with EVAL (split evaluation) they stay in shared memory and the block
+// evaluates them at its points (L2P, Eq. truncatedLE), adds the near-field
+// sums of k_near32 or k_near64 and writes the outputs.
 struct DownEval {
-  const float2 *loc;
+  const float2 *loc;   // single precision: leaf-frame positions, near sums
   const float4 *near;
+  const double *xs, *ys, *near64;  // double precision: positions, near sums [3][n]
+  int64_t n;
+  int *qexp;           // double precision: cleared for the next evaluation
   const int64_t *perm;
   const uint64_t *keys;  // sorted Morton keys: the leaf of each point
   const DevGeom *dg;
@@ -494,10 +515,14 @@ k_downward(int H, int k, int p, const cpx<R> *__restrict__ Tl2l, cpx<R> *__restr
   const int64_t lf0 = root << (2 * k);
   const int nl = 1 << (2 * k);
   const int i0 = leaf_start[lf0], i1 = leaf_start[lf0 + nl];
+  if constexpr (EVAL && sizeof(R) == 8) {
+    // (the near field, the charges' last reader by their exponent, is done)
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ev.qexp = 0;
+  }
   if (skip_empty && i1 == i0) return;  // a subtree without points needs no leaf expansions
   // with EVAL: the first point's data, loaded now, used after the L2L levels
   PointIn pf{};
-  if constexpr (EVAL) {
+  if constexpr (EVAL && sizeof(R) == 4) {
     if (i0 + (int)threadIdx.x < i1) pf = load_point(ev, i0 + (int)threadIdx.x);
   }
   A += blockIdx.y * rs.m;
@@ -635,7 +660,47 @@ k_downward(int H, int k, int p, const cpx<R> *__restrict__ Tl2l, cpx<R> *__restr
       np = nc;
     }
   }
-  if constexpr (EVAL) {
+  if constexpr (EVAL && sizeof(R) == 8) {
+    const double d = ev.dg->side / (double)(1 << H), invd = 1.0 / d;
+    const int ksh = 60 - 2 * H;
+    const double i2pi = 1.0 / HP_TWO_PI;
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+      const uint64_t leaf = ev.keys[i] >> ksh;
+      const int lo = (int)((int64_t)leaf - lf0);
+      const int ix = box_ix(leaf), iy = box_iy(leaf);
+      const cd *Al = reinterpret_cast<const cd *>(cur) + (size_t)lo * BS, *Bl = Al + P1;
+      const double2 c = leaf_centre_at(ev.dg->x0, d, ix, iy);
+      const cd w = mk((ev.xs[i] - c.x) * invd, (ev.ys[i] - c.y) * invd), wb = conj(w);
+      cd va = Al[p], da = mk(0.0, 0.0), vb = Bl[p], db = mk(0.0, 0.0);
+      for (int n = p - 1; n >= 0; --n) {
+        da = da * w + va;
+        va = va * w + Al[n];
+        db = db * wb + vb;
+        vb = vb * wb + Bl[n];
+      }
+      const double lf = ev.near64[i], fx = ev.near64[ev.n + i], fy = ev.near64[2 * ev.n + i];
+      cd u = va + vb, gx = invd * (da + db), gy = invd * (mul_i(da) - mul_i(db));
+      u.x = fma(-0.5 * i2pi, lf, u.x);
+      gx.x = fma(-i2pi, fx, gx.x);
+      gy.x = fma(-i2pi, fy, gy.x);
+      const int64_t o = ev.perm[i];
+      double2 *po = reinterpret_cast<double2 *>(ev.pot) + o;
+      double2 *go = reinterpret_cast<double2 *>(ev.grad) + 2 * o;
+      if (iy == 0) {  // bottom row: image/reaction sums already there
+        const double2 pm = *po;
+        u = u + mk(pm.x, pm.y);
+        if (ev.grad) {
+          gx = gx + mk(go[0].x, go[0].y);
+          gy = gy + mk(go[1].x, go[1].y);
+        }
+      }
+      *po = make_double2(u.x, u.y);
+      if (ev.grad) {
+        go[0] = make_double2(gx.x, gx.y);
+        go[1] = make_double2(gy.x, gy.y);
+      }
+    }
+  } else if constexpr (EVAL) {
     // L2P at the subtree's points (contiguous in tree order), plus the near
     // sums; cur holds the leaf expansions (when k = 0, the root's)
     const float invd = ev.dg->invd[H];
@@ -1128,95 +1193,6 @@ k_m2l_mirror_all(int H, int p, const DevGeom *__restrict__ dg, const cpx<R> *__r
   }
 }
 
-// --------------------------------------------------------------------------
-// Leaf evaluation: L2P of A and B (Eq. truncatedLE) plus the near field
-// (free part over the 3x3 neighbourhood, image and reaction parts over the
-// bottom-row neighbours), written in the caller's order.
-// One warp per leaf, lanes over 32 targets at a time; source points staged
-// per warp in shared memory.
-struct SrcPt64 { double x, y, q; };
-
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-k_eval64(const double *__restrict__ xs, const double *__restrict__ ys,
-         const double *__restrict__ qs, const int64_t *__restrict__ perm,
-         const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg, int p,
-         cd kappa, const cd *__restrict__ A, const cd *__restrict__ B, double *__restrict__ pot,
-         double *__restrict__ grad) {
-  __shared__ SrcPt64 sp[kWarpsPerBlock][32];
-  const double x0 = dg->x0, side = dg->side;
-  int P1 = p + 1;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int leaf = blockIdx.x * kWarpsPerBlock + warp;
-  int nx = 1 << H;
-  if (leaf >= nx * nx) return;
-  int ix = box_ix(leaf), iy = box_iy(leaf);
-  double d = side / (double)nx;
-  double cx = x0 + (ix + 0.5) * d, cy = (iy + 0.5) * d;
-  const cd *Al = A + (size_t)(level_offset(H) + leaf) * P1;
-  const cd *Bl = B + (size_t)(level_offset(H) + leaf) * P1;
-  int b0 = leaf_start[leaf], b1 = leaf_start[leaf + 1];
-  for (int tb = b0; tb < b1; tb += 32) {
-    int i = tb + lane;
-    bool act = i < b1;
-    double x = act ? xs[i] : cx, y = act ? ys[i] : cy;
-    // L2P: Horner for the value and the derivative in w and conj(w)
-    cd w = mk((x - cx) / d, (y - cy) / d), wb = conj(w);
-    cd va = Al[p], da = mk(0.0, 0.0), vb = Bl[p], db = mk(0.0, 0.0);
-    for (int n = p - 1; n >= 0; --n) {
-      da = da * w + va;
-      va = va * w + Al[n];
-      db = db * wb + vb;
-      vb = vb * wb + Bl[n];
-    }
-    cd u = va + vb;
-    cd gx = (1.0 / d) * (da + db);
-    cd gy = (1.0 / d) * (mul_i(da) - mul_i(db));
-    PairAcc<double> acc;
-    for (int ny = iy - 1; ny <= iy + 1; ++ny) {
-      if (ny < 0 || ny >= nx) continue;
-      for (int mxx = ix - 1; mxx <= ix + 1; ++mxx) {
-        if (mxx < 0 || mxx >= nx) continue;
-        uint64_t sl = box_morton(mxx, ny);
-        int s0 = leaf_start[sl], s1 = leaf_start[sl + 1];
-        bool mirror = (iy == 0 && ny == 0);
-        for (int sb = s0; sb < s1; sb += 32) {
-          __syncwarp();
-          int js = sb + lane;
-          if (js < s1) sp[warp][lane] = SrcPt64{xs[js], ys[js], qs[js]};
-          __syncwarp();
-          int cnt = min(32, s1 - sb);
-          if (!act) continue;
-          for (int k = 0; k < cnt; ++k) {
-            SrcPt64 s = sp[warp][k];
-            double dx = x - s.x;
-            if (sb + k != i) pair_free(acc, dx, y - s.y, s.q);
-            if (mirror) {
-              double Y = y + s.y;
-              pair_image(acc, dx, Y, s.q);
-              pair_reaction_d(acc, dx, Y, s.q, kappa);
-            }
-          }
-        }
-      }
-    }
-    if (!act) continue;
-    cd un, gxn, gyn;
-    acc.finish(un, gxn, gyn);
-    u = u + un;
-    gx = gx + gxn;
-    gy = gy + gyn;
-    int64_t o = perm[i];
-    pot[2 * o] = u.x;
-    pot[2 * o + 1] = u.y;
-    if (grad) {
-      grad[4 * o + 0] = gx.x;
-      grad[4 * o + 1] = gx.y;
-      grad[4 * o + 2] = gy.x;
-      grad[4 * o + 3] = gy.y;
-    }
-  }
-}
-
 // Single-precision leaf evaluation.  Coordinates are relative to the leaf
 // centre (exact leaf offsets are added per source leaf), so that the pair
 // differences keep full relative precision.  log via the SFU log2, the
@@ -1703,7 +1679,7 @@ k_eval_targets(const double *__restrict__ xt, const double *__restrict__ yt, int
                const double *__restrict__ xs, const double *__restrict__ ys,
                const float2 *__restrict__ loc, const R *__restrict__ qs,
                const int *__restrict__ leaf_start, int H, double x0, double side,
-               double qscale, int p, cd kappa, const cpx<R> *__restrict__ A,
+               double qscale, int p, KappaLog K, const cpx<R> *__restrict__ A,
                const cpx<R> *__restrict__ B, double *__restrict__ pot,
                double *__restrict__ grad) {
   const int lane = threadIdx.x & 31;
@@ -1799,8 +1775,7 @@ k_eval_targets(const double *__restrict__ xt, const double *__restrict__ yt, int
           }
           if (!kSingle && mirror) {
             const double ddx = hx - sxa, Y = hy + sya;
-            pair_image(ma, ddx, Y, (double)q);
-            pair_reaction_d(ma, ddx, Y, (double)q, kappa);
+            pair_mirror_d(ma, ddx, Y, (double)q, K);
           }
         }
       }
@@ -2054,14 +2029,16 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   }
   const DevGeom *dg = pl->dgeom;
 
-  // single precision, one RHS, the sources as targets: the free-space near
-  // field needs only the sorted points and charges, so it runs on this
-  // stream while the plan's side stream runs the far-field passes; L2P joins
-  // them
+  // one RHS, the sources as targets ("split"): the free-space near field
+  // needs only the sorted points and charges, so it runs on this stream while
+  // the plan's side stream runs the far-field passes; L2P joins them.  In
+  // double precision the near field takes the single-precision pipe (near64.cu)
+  // and the far field the FP64 pipe, so the two overlap.
   const int nxl = 1 << H, tps = nxl >= kTl ? nxl / kTl : 1;
-  const bool split = sizeof(R) == 4 && !mw && !tw;
-  if (split && !(pl->near && pl->side_stream && pl->ev_fork && pl->ev_join && pl->ev_gather)) {
-    set_last_error("single-precision plan without its near-field buffer or side stream");
+  const bool split = !mw && !tw;
+  if (split && !((sizeof(R) == 4 ? (void *)pl->near : (void *)pl->near64) && pl->side_stream &&
+                 pl->ev_fork && pl->ev_join && pl->ev_gather)) {
+    set_last_error("plan without its near-field buffer or side stream");
     return HPFMM_ECUDA;
   }
   // far-field chain: on the plan's high-priority side stream when split, so
@@ -2083,28 +2060,37 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   // near field reads them through perm itself)
   pass_begin(pl, fs, PASS_GATHER);
   if (split)
-    k_gather_q<R><<<dim3(cdiv_u(n, 256), nr), 256, 0, fs>>>(q, pl->perm, n, qs, (R *)nullptr, 0);
+    k_gather_q<R><<<dim3(cdiv_u(n, 256), nr), 256, 0, fs>>>(q, pl->perm, n, qs, (R *)nullptr, 0,
+                                                           pl->qexp);
   else
     HP_CUDA(launch_dependent(k_gather_q<R>, dim3(cdiv_u(n, 256), nr), dim3(256), 0, st, q,
-                             pl->perm, n, qs, mw ? (R *)mw->qsm : (R *)nullptr, mw ? mw->rp : 0));
+                             pl->perm, n, qs, mw ? (R *)mw->qsm : (R *)nullptr, mw ? mw->rp : 0,
+                             (int *)nullptr));
   pass_end(pl, fs, PASS_GATHER, 1);
   if (split) {
     HP_CUDA(cudaEventRecord(pl->ev_gather, fs));
+    if (sizeof(R) == 8) HP_CUDA(cudaStreamWaitEvent(st, pl->ev_gather, 0));
     pass_begin(pl, st, PASS_EVAL);
-    HP_CUDA(launch_dependent(k_near32, dim3((unsigned)(tps * tps)), dim3(32 * kEvWarps), kTpSmem,
-                             st, pl->loc32, pl->loclo, q, pl->perm,
-                             pl->leaf_start, H, dg, pl->near));
-    pass_end(pl, st, PASS_EVAL, 1);
+    if (sizeof(R) == 8)
+      HP_TRY(near64_launch(pl, (const double *)qs, st));
+    else
+      HP_CUDA(launch_dependent(k_near32, dim3((unsigned)(tps * tps)), dim3(32 * kEvWarps), kTpSmem,
+                               st, pl->loc32, pl->loclo, q, pl->perm,
+                               pl->leaf_start, H, dg, pl->near));
+    pass_end(pl, st, PASS_EVAL, sizeof(R) == 8 ? near64_kernels(pl) : 1);
     // the bottom-row image/reaction sums need only the sources too: written
     // now, added by the L2P kernel.  On the m2l stream (idle until the S2M is
     // done), off the near field's stream, after the gather.
     cudaStream_t ms = mirror_apart ? pl->m2l_stream : st;
     HP_CUDA(cudaStreamWaitEvent(ms, pl->ev_gather, 0));
     pass_begin(pl, ms, PASS_NEAR_MIRROR);
-    k_mirror32<<<dim3((unsigned)(1 << H), 1, kMirSplit), 32 * kEvWarps, 0, ms>>>(
-        pl->loc32, pl->yabs, (const float *)qs, pl->perm, pl->leaf_start, H, dg,
-        kappa_log(pl->kre, pl->kim), pl->prec == HPFMM_MIXED ? (float)pl->tau_fp64 : 0.f, pot,
-        grad, rs, 1);
+    if (sizeof(R) == 8)
+      HP_TRY(mirror64_launch(pl, (const double *)qs, pot, grad, ms));
+    else
+      k_mirror32<<<dim3((unsigned)(1 << H), 1, kMirSplit), 32 * kEvWarps, 0, ms>>>(
+          pl->loc32, pl->yabs, (const float *)qs, pl->perm, pl->leaf_start, H, dg,
+          kappa_log(pl->kre, pl->kim), pl->prec == HPFMM_MIXED ? (float)pl->tau_fp64 : 0.f, pot,
+          grad, rs, 1);
     pass_end(pl, ms, PASS_NEAR_MIRROR, 1);
   }
   pass_begin(pl, fs, PASS_P2M);
@@ -2236,14 +2222,15 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   // after the near field has joined, the same kernel evaluates the leaf
   // expansions at the points (on the caller's stream); otherwise the leaf
   // expansions go to memory for the leaf kernels below.
-  const DownEval noev{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  const DownEval noev{};
   if (split) {
     HP_CUDA(cudaEventRecord(pl->ev_join, fs));
     HP_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
     int kd = H - 1 < 3 ? H - 1 : 3;  // subtrees of 64 leaves: 4^(H-3) blocks
     while (kd > 0 && downward_smem<R>(p, kd, true) > kFusedSmem) --kd;
     pass_begin(pl, st, PASS_L2L);
-    const DownEval ev{pl->loc32, pl->near, pl->perm, pl->keys, dg, pot, grad};
+    const DownEval ev{pl->loc32, pl->near, pl->xs,  pl->ys, pl->near64, n, pl->qexp,
+                      pl->perm,  pl->keys, dg, pot, grad};
     k_downward<R, true><<<dim3((unsigned)(int64_t(1) << (2 * (H - kd))), 1), 256,
                           downward_smem<R>(p, kd, true), st>>>(
         H, kd, p, Tl2l, A, B, rs, pl->leaf_start, 1, ev,
@@ -2262,12 +2249,11 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   pass_end(pl, fs, PASS_L2L, ksub > 0 ? 1 : 0);
   pass_begin(pl, st, PASS_EVAL);
   // evaluation at the leaves + near field
-  cd kappa = mk(pl->kre, pl->kim);
   if (tw) {
     if (tw->nt > 0)
       k_eval_targets<R><<<cdiv_u(tw->nt, 256), 256, 0, st>>>(
           tw->xt, tw->yt, tw->nt, pl->xs, pl->ys, pl->loc32, (const R *)qs, pl->leaf_start, H,
-          pl->x0, pl->side, pl->qscale, p, kappa, A, B, pot, grad);
+          pl->x0, pl->side, pl->qscale, p, kappa_log(pl->kre, pl->kim), A, B, pot, grad);
     pass_end(pl, st, PASS_EVAL, tw->nt > 0 ? 1 : 0);
     if (sizeof(R) == 4 && tw->nbottom > 0) {
       pass_begin(pl, st, PASS_NEAR_MIRROR);
@@ -2280,21 +2266,16 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
     HP_LAUNCH_CHECK();
     return HPFMM_OK;
   }
-  if (sizeof(R) == 8) {
-    k_eval64<<<cdiv_u(pl->nleaf, kWarpsPerBlock), 32 * kWarpsPerBlock, 0, st>>>(
-        pl->xs, pl->ys, (const double *)qs, pl->perm, pl->leaf_start, H, dg, p,
-        kappa, (const cd *)A, (const cd *)B, pot, grad);
-  } else {
-    float tau = pl->prec == HPFMM_MIXED ? (float)pl->tau_fp64 : 0.f;
-    if (mw) {
-      k_eval32m<kRhsChunk><<<dim3(cdiv_u(pl->nleaf, kEvWarps), mw->rp / kRhsChunk),
-                             32 * kEvWarps, 0, st>>>(
-          pl->loc32, (const float *)mw->qsm, mw->rp, nr, pl->perm, pl->leaf_start, H, dg, p,
-          (const cf *)A, (const cf *)B, rs, pot, grad);
-    } else {
-      set_last_error("single-RHS single-precision evaluation outside the split path");
-      return HPFMM_ECUDA;
-    }
+  if (!mw) {
+    set_last_error("single-RHS evaluation outside the split path");
+    return HPFMM_ECUDA;
+  }
+  if constexpr (sizeof(R) == 4) {
+    const float tau = pl->prec == HPFMM_MIXED ? (float)pl->tau_fp64 : 0.f;
+    k_eval32m<kRhsChunk><<<dim3(cdiv_u(pl->nleaf, kEvWarps), mw->rp / kRhsChunk), 32 * kEvWarps, 0,
+                           st>>>(pl->loc32, (const float *)mw->qsm, mw->rp, nr, pl->perm,
+                                 pl->leaf_start, H, dg, p, (const cf *)A, (const cf *)B, rs, pot,
+                                 grad);
     pass_end(pl, st, PASS_EVAL, 1);
     pass_begin(pl, st, PASS_NEAR_MIRROR);
     k_mirror32<<<dim3((unsigned)(1 << H), nr, kMirSplit), 32 * kEvWarps, 0, st>>>(
@@ -2302,7 +2283,6 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
         kappa_log(pl->kre, pl->kim), tau, pot, grad, rs, 0);
     pass_end(pl, st, PASS_NEAR_MIRROR, 1);
   }
-  if (sizeof(R) == 8) pass_end(pl, st, PASS_EVAL, 1);
   HP_LAUNCH_CHECK();
   return HPFMM_OK;
 }
@@ -2330,6 +2310,8 @@ hpfmm_status fmm_set_smem_limits(int p) {
   HP_CUDA(cudaFuncSetAttribute(k_downward<double, false>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));
   HP_CUDA(cudaFuncSetAttribute(k_downward<float, false>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));
+  HP_CUDA(cudaFuncSetAttribute(k_downward<double, true>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));
   HP_CUDA(cudaFuncSetAttribute(k_downward<float, true>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));

@@ -61,10 +61,11 @@ __device__ __forceinline__ void mirror_pair(const float4 s, float mx, float my, 
   } else {
     const double X = dx, Yd = Y;
     cd J0p, J1p, J0m, J1m;
-    j01_pm(K, X, Yd, J0p, J1p, J0m, J1m);
+    const double s2 = X * X + Yd * Yd;
+    j01_pm(K, X, Yd, s2, log(s2), J0p, J1p, J0m, J1m);
     const double q = s.z;
     // J_1 / s+- with s+- = Y -+ iX: one reciprocal of |s|^2 for both
-    const double inv = 1.0 / (X * X + Yd * Yd);
+    const double inv = 1.0 / s2;
     const cd tp = inv * (J1p * mk(Yd, X)), tm = inv * (J1m * mk(Yd, -X));
     a.ur = a.ur + to<float>(q * (J0p + J0m));
     a.grx = a.grx + to<float>(q * mul_i(tp - tm));

@@ -38,25 +38,19 @@ __device__ __forceinline__ void pair_free(PairAcc<R> &a, R dx, R dy, R q) {
   a.gfy += qi * dy;
 }
 
-template <typename R>
-__device__ __forceinline__ void pair_image(PairAcc<R> &a, R dx, R Y, R q) {
-  R r2 = dx * dx + Y * Y;
-  R inv = R(1) / r2;
-  a.li += q * log(r2);
-  R qi = q * inv;
-  a.gix += qi * dx;
+// image and reaction pair in double precision: |s|^2 = X^2 + Y^2, its log and
+// its reciprocal serve both (J_1 / s+- with s+- = Y -+ iX)
+__device__ __forceinline__ void pair_mirror_d(PairAcc<double> &a, double X, double Y, double q,
+                                              const KappaLog &K) {
+  const double s2 = X * X + Y * Y, ln = log(s2), inv = 1.0 / s2;
+  a.li += q * ln;
+  const double qi = q * inv;
+  a.gix += qi * X;
   a.giy += qi * Y;
-}
-
-// reaction pair in double precision
-__device__ __forceinline__ void pair_reaction_d(PairAcc<double> &a, double dx, double Y,
-                                                double q, cd kappa) {
-  cd sp = mk(Y, -dx), sm = mk(Y, dx);
   cd J0p, J1p, J0m, J1m;
-  j01(kappa * sp, J0p, J1p);
-  j01(kappa * sm, J0m, J1m);
+  j01_pm(K, X, Y, s2, ln, J0p, J1p, J0m, J1m);
   a.ur = a.ur + q * (J0p + J0m);
-  cd tp = cdiv(J1p, sp), tm = cdiv(J1m, sm);
-  a.grx = a.grx + q * mul_i(tp - tm);
-  a.gry = a.gry - q * (tp + tm);
+  const cd tp = J1p * mk(Y, X), tm = J1m * mk(Y, -X);
+  a.grx = a.grx + qi * mul_i(tp - tm);
+  a.gry = a.gry - qi * (tp + tm);
 }

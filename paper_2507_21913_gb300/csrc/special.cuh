@@ -39,6 +39,13 @@
 // special_init_here() fills it once per device.
 constexpr int kRecip = 512;
 static __constant__ double c_recip[kRecip];
+// Coefficients of the J_0 and J_1 power series (j01_arg), c_ser[0][k] = 1/(k k!)
+// and c_ser[1][k] = 1/((k-1) k!), and the terms they need: c_nser[i] for
+// |P| <= (i + 1) / 4 (a^N / N! <= 1e-17 max(1, a^2), well below the rounding of
+// the sum).
+constexpr int kSer = 64, kNser = 16;
+static __constant__ double c_ser[2][kSer];
+static __constant__ int c_nser[kNser];
 static inline hpfmm_status special_init_here() {
   static std::mutex mu;
   static bool done[64] = {};
@@ -54,6 +61,23 @@ static inline hpfmm_status special_init_here() {
   host[0] = 0.0;
   for (int k = 1; k < kRecip; ++k) host[k] = 1.0 / (double)k;
   HP_CUDA(cudaMemcpyToSymbol(c_recip, host, sizeof host));
+  static double ser[2][kSer];
+  static int nser[kNser];
+  double f = 1.0;  // k!
+  for (int k = 0; k < kSer; ++k) {
+    if (k > 1) f *= (double)k;
+    ser[0][k] = k > 0 ? 1.0 / ((double)k * f) : 0.0;
+    ser[1][k] = k > 1 ? 1.0 / ((double)(k - 1) * f) : 0.0;
+  }
+  for (int i = 0; i < kNser; ++i) {
+    const double a = 0.25 * (i + 1);
+    double t = 1.0;
+    int k = 0;
+    while (k < kSer - 1 && (k < a || t > 1e-18)) t *= a / (double)++k;
+    nser[i] = k;
+  }
+  HP_CUDA(cudaMemcpyToSymbol(c_ser, ser, sizeof ser));
+  HP_CUDA(cudaMemcpyToSymbol(c_nser, nser, sizeof nser));
   done[dev] = true;
   return HPFMM_OK;
 }
@@ -146,39 +170,6 @@ __device__ inline cd jn_direct_single(cd P, int n) {
   return series ? jn_series(P, n) : jn_cf(P, n);
 }
 
-// J_0 and J_1 = 1 + P J_0 for |P| <= 1/8, double precision: the series form
-// of J_0 above, J_0 = e^{-P}[i pi - gamma - Log P - sum_{k>=1} P^k/(k k!)],
-// with e^{-P} and the sum as fixed-length polynomials in P (Horner).  At
-// |P| = 1/8 the first dropped terms are below 3e-18 relative.  Near-field
-// reaction pairs next to the boundary have |P| of a few leaf sides, so this
-// replaces a complex exponential and a loop of the general series there.
-__device__ __forceinline__ void j01_small(cd P, cd &J0, cd &J1) {
-  // sum_{k=1}^{10} P^k / (k k!)
-  cd S = mk(1.0 / (10.0 * 3628800.0), 0.0);
-  const double cs[9] = {1.0, 1.0 / 4.0, 1.0 / 18.0, 1.0 / 96.0, 1.0 / 600.0, 1.0 / 4320.0,
-                        1.0 / 35280.0, 1.0 / 322560.0, 1.0 / 3265920.0};
-#pragma unroll
-  for (int k = 8; k >= 0; --k) {
-    S = S * P;
-    S.x += cs[k];
-  }
-  S = S * P;
-  // e^{-P} = sum_{k=0}^{10} (-P)^k / k!
-  const cd mP = mk(-P.x, -P.y);
-  const double ce[10] = {1.0, 1.0, 1.0 / 2.0, 1.0 / 6.0, 1.0 / 24.0, 1.0 / 120.0,
-                         1.0 / 720.0, 1.0 / 5040.0, 1.0 / 40320.0, 1.0 / 362880.0};
-  cd E = mk(1.0 / 3628800.0, 0.0);
-#pragma unroll
-  for (int k = 9; k >= 0; --k) {
-    E = E * mP;
-    E.x += ce[k];
-  }
-  const double lr = 0.5 * log(abs2(P)), th = atan2(P.y, P.x);
-  J0 = E * mk(-HP_EULER_GAMMA - lr - S.x, HP_PI - th - S.y);
-  const cd v = P * J0;
-  J1 = mk(1.0 + v.x, v.y);
-}
-
 // kappa with its logarithm ln|kappa| + i arg kappa, computed once on the host
 struct KappaLog {
   cd kappa;
@@ -192,76 +183,146 @@ inline KappaLog kappa_log(double kre, double kim) {
   return K;
 }
 
-__device__ inline void j01(cd P, cd &J0, cd &J1);
-
-// e^{-P} and sum_{k>=1} P^k/(k k!) by Horner, N + 1 and N terms (N <= 10)
+// sum_{k=0}^{N-1} c[k] z^k for real coefficients and complex z by the real
+// recurrence b_k = c_k + 2 Re(z) b_{k+1} - |z|^2 b_{k+2} (the quotient of the
+// polynomial by z^2 - 2 Re(z) z + |z|^2): two FP64 instructions a term, where
+// Horner's rule in complex arithmetic takes four.
 template <int N>
-__device__ __forceinline__ void exp_sum_poly(cd P, cd &E, cd &S) {
+__device__ __forceinline__ cd real_poly(const double (&c)[N], cd z, double z2) {
+  double b1 = c[N - 1], b2 = 0.0;
+  const double r = z.x + z.x;
+#pragma unroll
+  for (int k = N - 2; k >= 1; --k) {
+    const double t = fma(r, b1, fma(-z2, b2, c[k]));
+    b2 = b1;
+    b1 = t;
+  }
+  return mk(fma(z.x, b1, fma(-z2, b2, c[0])), z.y * b1);
+}
+
+// e^{-P} and sum_{k>=1} P^k/(k k!) to P^N, P2 = |P|^2 (N <= 10)
+template <int N>
+__device__ __forceinline__ void exp_sum_poly(cd P, double P2, cd &E, cd &S) {
   const double ce[11] = {1.0, 1.0, 1.0 / 2.0, 1.0 / 6.0, 1.0 / 24.0, 1.0 / 120.0, 1.0 / 720.0,
                          1.0 / 5040.0, 1.0 / 40320.0, 1.0 / 362880.0, 1.0 / 3628800.0};
   const double cs[11] = {0.0, 1.0, 1.0 / 4.0, 1.0 / 18.0, 1.0 / 96.0, 1.0 / 600.0,
                          1.0 / 4320.0, 1.0 / 35280.0, 1.0 / 322560.0, 1.0 / 3265920.0,
                          1.0 / 36288000.0};
-  const cd mP = mk(-P.x, -P.y);
-  E = mk(ce[N], 0.0);
-  S = mk(cs[N], 0.0);
+  double e[N], s[N];
 #pragma unroll
-  for (int k = N - 1; k >= 1; --k) {
-    E = E * mP;
-    E.x += ce[k];
-    S = S * P;
-    S.x += cs[k];
+  for (int k = 0; k < N; ++k) {
+    e[k] = ce[k + 1];
+    s[k] = cs[k + 1];
   }
-  E = E * mP;
+  const cd mP = mk(-P.x, -P.y);
+  E = mP * real_poly<N>(e, mP, P2);
   E.x += 1.0;
-  S = S * P;
+  S = P * real_poly<N>(s, P, P2);
+}
+
+// J_0 and J_1 of one argument, |P| = a, given Log P = lr + i arg and e^{-P}: the
+// power series where it does not cancel (the region of jn_use_series), J_0
+// below |P| = 1 and J_1 above (where 1 + P J_0 would cancel), each with
+// J_1 = 1 + P J_0 for the other; the general forms elsewhere (beyond |P| = 4 the
+// recurrence of real_poly would lose about |P| of the series' precision).
+__device__ __forceinline__ void j01_arg(cd P, double P2, float a, double lr, double arg, cd E,
+                                        cd &J0, cd &J1) {
+  const bool big = P2 >= 1.0;
+  if (a <= 0.5f || (a <= 4.0f && (double)a - P.x <= 1.5)) {
+    // the lanes take one term count: the coefficients are read uniformly
+    const int N = __reduce_max_sync(__activemask(), c_nser[min((int)(4.0f * a), kNser - 1)]);
+    const double r = P.x + P.x;
+    double b1 = 0.0, b2 = 0.0;
+    if (!big) {
+      for (int k = N; k >= 2; --k) {
+        const double t = fma(r, b1, fma(-P2, b2, c_ser[0][k]));
+        b2 = b1;
+        b1 = t;
+      }
+      // sum_{k>=1} c_k P^(k-1)
+      const cd S = P * mk(fma(P.x, b1, fma(-P2, b2, 1.0)), P.y * b1);
+      J0 = E * mk(-HP_EULER_GAMMA - lr - S.x, HP_PI - arg - S.y);
+      const cd v = P * J0;
+      J1 = mk(1.0 + v.x, v.y);
+      return;
+    }
+    for (int k = N; k >= 3; --k) {
+      const double t = fma(r, b1, fma(-P2, b2, c_ser[1][k]));
+      b2 = b1;
+      b1 = t;
+    }
+    // P sum_{k>=2} c_k P^(k-2), c_2 = 1/2, and the log terms
+    const cd T = P * mk(fma(P.x, b1, fma(-P2, b2, 0.5)), P.y * b1);
+    cd v = P * mk(1.0 - HP_EULER_GAMMA - lr - T.x, HP_PI - arg - T.y);
+    v.x += 1.0;
+    J1 = E * v;
+  } else if (!big) {
+    J0 = jn_cf(P, 0);
+    const cd v = P * J0;
+    J1 = mk(1.0 + v.x, v.y);
+    return;
+  } else {
+    J1 = jn_direct(P, 1);
+  }
+  const double inv = 1.0 / P2;
+  J0 = inv * (mk(P.x, -P.y) * mk(J1.x - 1.0, J1.y));
 }
 
 // J_0 and J_1 of both reaction arguments of one pair, P+ = kappa (Y - iX) and
-// P- = kappa (Y + iX) (Y > 0), double precision.  For |P| <= 1/8 the series
-// of j01_small, with Log P+- = Log kappa + ln|s| -+ i atan2(X, Y) (s+- = Y -+
-// iX are conjugate, and the sum of the arguments stays in (-pi/2, pi)), so
-// that one log and one atan2 serve both; 6 terms for |P| <= 1/64, 11 above
-// (dropped terms below 1e-16 relative).  Larger |P|: j01 twice.
-__device__ __forceinline__ void j01_pm(const KappaLog &K, double X, double Y, cd &J0p, cd &J1p,
-                                       cd &J0m, cd &J1m) {
+// P- = kappa (Y + iX) (Y > 0), double precision, s2 = X^2 + Y^2 and its log
+// given (the image term of the pair needs both).  Log P+- = Log kappa + ln|s|
+// -+ i atan2(X, Y) (s+- = Y -+ iX are conjugate, and the sum of the arguments
+// stays in (-pi/2, pi)), so one log and one atan2 serve both.  For |P| <= 1/8
+// fixed-length series: 6 terms for |P| <= 1/64, 10 above (dropped terms below
+// 1e-16 relative).  Beyond, j01_arg.  For real kappa the two arguments are
+// conjugate and J_n(conj P) = conj J_n(P) + 2 pi i conj(P)^n e^{-conj P}
+// (only the i pi of the seed is not conjugated): one evaluation, at the
+// argument with Im P >= 0, whose value holds no residue term to cancel.
+// FP64 instructions a pair, beside log and atan2: about 60 for |P| <= 1/8
+// with real kappa, 200 for |P| about 1 (the series of each argument by complex
+// Horner steps and a term-by-term test took about 250 and 1500).
+__device__ __forceinline__ void j01_pm(const KappaLog &K, double X, double Y, double s2,
+                                       double ln_s2, cd &J0p, cd &J1p, cd &J0m, cd &J1m) {
   const cd Pp = K.kappa * mk(Y, -X), Pm = K.kappa * mk(Y, X);
-  const double s2 = X * X + Y * Y, a2 = abs2(K.kappa) * s2;
-  if (a2 > 1.0 / 64.0) {
-    j01(Pp, J0p, J1p);
-    j01(Pm, J0m, J1m);
+  const double a2 = abs2(K.kappa) * s2;
+  const double lr = fma(0.5, ln_s2, K.lk), th = atan2(X, Y);
+  const bool real = K.kappa.y == 0.0;
+  if (a2 <= 1.0 / 64.0) {
+    cd Ep, Sp, Em, Sm;
+    if (a2 <= 1.0 / 4096.0) {
+      exp_sum_poly<6>(Pp, a2, Ep, Sp);
+      if (!real) exp_sum_poly<6>(Pm, a2, Em, Sm);
+    } else {
+      exp_sum_poly<10>(Pp, a2, Ep, Sp);
+      if (!real) exp_sum_poly<10>(Pm, a2, Em, Sm);
+    }
+    if (real) {
+      Em = conj(Ep);
+      Sm = conj(Sp);
+    }
+    J0p = Ep * mk(-HP_EULER_GAMMA - lr - Sp.x, HP_PI - (K.ak - th) - Sp.y);
+    J0m = Em * mk(-HP_EULER_GAMMA - lr - Sm.x, HP_PI - (K.ak + th) - Sm.y);
+    const cd vp = Pp * J0p, vm = Pm * J0m;
+    J1p = mk(1.0 + vp.x, vp.y);
+    J1m = mk(1.0 + vm.x, vm.y);
     return;
   }
-  const double lr = K.lk + 0.5 * log(s2), th = atan2(X, Y);
-  cd Ep, Sp, Em, Sm;
-  if (a2 <= 1.0 / 4096.0) {
-    exp_sum_poly<6>(Pp, Ep, Sp);
-    exp_sum_poly<6>(Pm, Em, Sm);
+  const float a = sqrtf((float)a2);
+  if (real) {
+    const bool up = X > 0.0;  // P- has Im >= 0
+    const cd P = up ? Pm : mk(Pp.x, Pp.y);
+    const cd E = cexp_d(-P), Ec = conj(E);
+    cd J0, J1;
+    j01_arg(P, a2, a, lr, fabs(th), E, J0, J1);
+    const cd r0 = HP_TWO_PI * mul_i(Ec), r1 = conj(P) * r0;
+    const cd Q0 = conj(J0) + r0, Q1 = conj(J1) + r1;
+    J0m = up ? J0 : Q0;
+    J1m = up ? J1 : Q1;
+    J0p = up ? Q0 : J0;
+    J1p = up ? Q1 : J1;
   } else {
-    exp_sum_poly<10>(Pp, Ep, Sp);
-    exp_sum_poly<10>(Pm, Em, Sm);
-  }
-  J0p = Ep * mk(-HP_EULER_GAMMA - lr - Sp.x, HP_PI - (K.ak - th) - Sp.y);
-  J0m = Em * mk(-HP_EULER_GAMMA - lr - Sm.x, HP_PI - (K.ak + th) - Sm.y);
-  const cd vp = Pp * J0p, vm = Pm * J0m;
-  J1p = mk(1.0 + vp.x, vp.y);
-  J1m = mk(1.0 + vm.x, vm.y);
-}
-
-// J_0 and J_1 = 1 + P J_0 (direct and near-field kernels), double precision
-__device__ inline void j01(cd P, cd &J0, cd &J1) {
-  double a = sqrt(abs2(P));
-  if (a <= 0.125) {
-    j01_small(P, J0, J1);
-  } else if (a < 1.0) {
-    J0 = jn_direct(P, 0);
-    cd v = P * J0;
-    J1 = mk(1.0 + v.x, v.y);
-  } else {
-    // 1 + P J_0 cancels for large |P|: evaluate J_1 directly and take one
-    // downward step of the recursion (stable for n <= |P|)
-    J1 = jn_direct(P, 1);
-    J0 = cinv(P) * mk(J1.x - 1.0, J1.y);
+    j01_arg(Pp, a2, a, lr, K.ak - th, cexp_d(-Pp), J0p, J1p);
+    j01_arg(Pm, a2, a, lr, K.ak + th, cexp_d(-Pm), J0m, J1m);
   }
 }
 
