@@ -196,11 +196,11 @@ def vlist_translations(H):
 # the dominant-kernel roofline); a pass may take several launches per step (the
 # leaf-level M2L runs apart from the coarser levels, the tree build is six
 # kernels), and its work per launch is then the step's work over its launches
-PASS_KERNELS = {"eval": ("k_near32", "k_eval64"), "m2l_free": ("k_m2l_free_patch", None),
+PASS_KERNELS = {"eval": ("k_near32", "k_near64"), "m2l_free": ("k_m2l_free_patch", None),
                 "m2l_mirror": ("k_m2l_mirror_all", "k_m2l_mirror_all"),
-                "p2m": ("k_s2m_tile", "k_p2m"), "near_mirror": ("k_mirror32", None),
+                "p2m": ("k_s2m_tile", "k_p2m64"), "near_mirror": ("k_mirror32", "k_mirror64"),
                 "tree": ("k_tb_* (tree build: bbox, keys, scan, scatter, sort, big-leaf sort)",) * 2,
-                "l2l": ("k_downward<float, true>", "k_downward<double, false>")}
+                "l2l": ("k_downward<float, true>", "k_downward<double, true>")}
 
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a

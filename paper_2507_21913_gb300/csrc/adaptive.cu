@@ -544,8 +544,8 @@ k_ad_mirror(int bfirst, int blast, int nbox, int p, AdGeom g, const cf *__restri
       const int dx = ixs - ixt, ysum = iyt + iys + 1;
       const int cls = (ysum - 1) * 7 + (dx + 3);
       const cf mine = lane < P1 ? M[(size_t)s * P1 + lane] : mk(0.f, 0.f);
-      const cf *Ti = Timg + (size_t)cls * P1 * P1 + (size_t)row * P1;
-      const cf *Tp = Treact + ((size_t)((l - 1) * 21 + cls) * 2) * P1 * P1 + (size_t)row * P1;
+      const cf *Ti = Timg + (size_t)cls * P1 * P1 + row;
+      const cf *Tp = Treact + ((size_t)((l - 1) * 21 + cls) * 2) * P1 * P1 + row;
       const cf *Tm = Tp + (size_t)P1 * P1;
       for (int kk = 0; kk < P1; ++kk) {
         cf mv;
@@ -553,9 +553,9 @@ k_ad_mirror(int bfirst, int blast, int nbox, int p, AdGeom g, const cf *__restri
         mv.y = __shfl_sync(0xffffffffu, mine.y, kk);
         if (lane < P1) {
           const cf mc = conj(mv);
-          cfma(aL, Ti[kk], mc);
-          cfma(aC, Tp[kk], mc);
-          cfma(aD, Tm[kk], mv);
+          cfma(aL, Ti[kk * P1], mc);
+          cfma(aC, Tp[kk * P1], mc);
+          cfma(aD, Tm[kk * P1], mv);
         }
       }
       const float m0 = __shfl_sync(0xffffffffu, mine.x, 0);
@@ -698,8 +698,7 @@ k_ad_eval(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
     const float2 mel = act ? loclo[i] : make_float2(0.f, 0.f);
     f2p gsum = f2_pack(0.f, 0.f);
     NearAcc a;
-    a.lf = a.gx = a.gy = a.li = a.gix = a.giy = 0.f;
-    a.ur = a.grx = a.gry = mk(0.f, 0.f);
+    a.lf = a.gx = a.gy = 0.f;
     // leaves at level >= l inside the 3 x 3 cells around D
     for (unsigned mA = maskA; mA; mA &= mA - 1) {
       const int jc = __ffs(mA) - 1;
@@ -744,12 +743,7 @@ k_ad_eval(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
     const cf *Bl = B + (size_t)D * P1;
     const cf w = mk(me.x * invd, me.y * invd), wb = conj(w);
     cf va = Al[p], da = mk(0.f, 0.f), vb = Bl[p], db = mk(0.f, 0.f);
-    for (int n = p - 1; n >= 0; --n) {
-      da = da * w + va;
-      va = va * w + Al[n];
-      db = db * wb + vb;
-      vb = vb * wb + Bl[n];
-    }
+    for (int n = p - 1; n >= 0; --n) horner4(va, da, vb, db, w, wb, Al[n], Bl[n]);
     const float ur = va.x + vb.x - a.lf * c4;
     const float ui = va.y + vb.y;
     const cf gxo = invd * (da + db) + mk(-a.gx * i2pi, 0.f);
@@ -803,16 +797,13 @@ k_ad_mirror_near(const float2 *__restrict__ loc, const float *__restrict__ yabs,
   }
   const unsigned maskB = __ballot_sync(0xffffffffu, cb >= 0);
   if (!maskA && !maskB) return;
-  const cf kap = mk((float)K.kappa.x, (float)K.kappa.y);
-  const float c4 = (float)(0.69314718055994530942 / (4.0 * HP_PI));
-  const float i2pi = (float)(1.0 / HP_TWO_PI);
+  const KappaF kf = kappa_f(K);
   for (int tb = lo[D]; tb < hi[D]; tb += 32) {
     const int i = tb + lane;
     const bool act = i < hi[D];
     const float mx = act ? loc[i].x : 0.f, my = act ? yabs[i] : 0.f;
-    NearAcc a;
-    a.lf = a.gx = a.gy = a.li = a.gix = a.giy = 0.f;
-    a.ur = a.grx = a.gry = mk(0.f, 0.f);
+    MirrorAcc a;
+    a.clear();
     for (unsigned m = maskA; m; m &= m - 1) {
       const int nb = __shfl_sync(0xffffffffu, nbA, __ffs(m) - 1);
       const int r1 = min(rank[hi[nb]], nleaf);
@@ -822,8 +813,7 @@ k_ad_mirror_near(const float2 *__restrict__ loc, const float *__restrict__ yabs,
         const float ox = ad_offset(g, lvl[C], box_ix(kC), box_iy(kC), l, ix, iy).x;
         if (act)
           for (int kk = lo[C]; kk < hi[C]; ++kk)
-            mirror_pair(make_float4(loc[kk].x + ox, yabs[kk], qs[kk], 0.f), mx, my, kap, K, tau,
-                        a);
+            a.add(qs[kk], mirror_value(mx - (loc[kk].x + ox), my + yabs[kk], kf, K, tau));
       }
     }
     for (unsigned m = maskB; m; m &= m - 1) {
@@ -833,18 +823,9 @@ k_ad_mirror_near(const float2 *__restrict__ loc, const float *__restrict__ yabs,
       const float ox = ad_offset(g, la, (ix >> (l - la)) + dx, 0, l, ix, iy).x;
       if (act)
         for (int kk = lo[C]; kk < hi[C]; ++kk)
-          mirror_pair(make_float4(loc[kk].x + ox, yabs[kk], qs[kk], 0.f), mx, my, kap, K, tau, a);
+          a.add(qs[kk], mirror_value(mx - (loc[kk].x + ox), my + yabs[kk], kf, K, tau));
     }
-    if (!act) continue;
-    const int64_t o = perm[i];
-    pot[2 * o] += (double)(a.li * c4 + a.ur.x * i2pi);
-    pot[2 * o + 1] += (double)(a.ur.y * i2pi);
-    if (grad) {
-      grad[4 * o + 0] += (double)((a.gix + a.grx.x) * i2pi);
-      grad[4 * o + 1] += (double)(a.grx.y * i2pi);
-      grad[4 * o + 2] += (double)((a.giy + a.gry.x) * i2pi);
-      grad[4 * o + 3] += (double)(a.gry.y * i2pi);
-    }
+    if (act) a.put(pot, grad, perm[i], false);
   }
 }
 

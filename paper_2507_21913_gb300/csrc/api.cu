@@ -461,7 +461,7 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
   if (f32) ALLOC(pl->yabs, sizeof(float) * n);
   if (f32) ALLOC(pl->loclo, sizeof(float2) * n);
   if (f32 && !pl->adaptive) ALLOC(pl->near, sizeof(float4) * n);
-  if (!pl->adaptive) {  // mirror M2L results: rows 0 and 1 of levels 1..H
+  if (f32 && !pl->adaptive) {  // mirror M2L results: rows 0 and 1 of levels 1..H
     ALLOC(pl->mir_A, csz * 4 * (((size_t)1 << pl->H) - 1) * P1);
     ALLOC(pl->mir_B, csz * 4 * (((size_t)1 << pl->H) - 1) * P1);
   }
@@ -501,6 +501,7 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
   if (s == HPFMM_OK) s = fmm_prepare();
   if (s == HPFMM_OK) s = adaptive_prepare();
   if (s == HPFMM_OK) s = near64_prepare();
+  if (s == HPFMM_OK) s = tables_prepare();
   if (s != HPFMM_OK) { free_plan(pl); return s; }
   {
     // the far-field streams of a split evaluation -- side (S2M, M2M, coarse

@@ -66,6 +66,23 @@ __host__ __device__ __forceinline__ void cfma(cpx<R> &a, cpx<R> b, cpx<R> c) {
   a.x = fma(b.x, c.x, fma(-b.y, c.y, a.x));
   a.y = fma(b.x, c.y, fma(b.y, c.x, a.y));
 }
+// one Horner step of an analytic and an anti-analytic expansion (values va, vb
+// in w and conj w, derivatives da, db): four multiply-adds a product
+template <typename R>
+__device__ __forceinline__ void horner4(cpx<R> &va, cpx<R> &da, cpx<R> &vb, cpx<R> &db, cpx<R> w,
+                                        cpx<R> wb, cpx<R> a, cpx<R> b) {
+  cpx<R> ta = va, tb = vb;
+  cfma(ta, da, w);
+  cfma(tb, db, wb);
+  da = ta;
+  db = tb;
+  ta = a;
+  tb = b;
+  cfma(ta, va, w);
+  cfma(tb, vb, wb);
+  va = ta;
+  vb = tb;
+}
 template <typename R>
 __host__ __device__ __forceinline__ cpx<R> cinv(cpx<R> b) {
   // 1/b = conj(b')/|b'|^2 * (1/s) with b' = b/s, s = |re| + |im| (no overflow);
@@ -272,6 +289,17 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// The kernels of an evaluation run beside one another, and an SM changes its
+// split between L1 and shared memory only when it is idle: a kernel that wants
+// more shared memory than the split of the kernel it runs beside leaves waits
+// for that one's blocks to end.  So they all ask for the largest shared-memory
+// split.
+template <typename F>
+cudaError_t prefer_shared(F *kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                              cudaSharedmemCarveoutMaxShared);
 }
 
 // centre of leaf (ix, iy) of side d in the root square starting at x0, with
@@ -488,6 +516,7 @@ hpfmm_status adaptive_alloc(hpfmm_plan *pl);
 // stream capture such as the batched graph)
 hpfmm_status fmm_prepare();
 hpfmm_status near64_prepare();
+hpfmm_status tables_prepare();
 // near field of a double-precision plan (near64.cu): the free-space pair sums
 // to pl->near64, the bottom row's image and reaction pairs to the outputs
 hpfmm_status near64_launch(hpfmm_plan *pl, const double *qs, cudaStream_t st);

@@ -48,15 +48,12 @@ constexpr int kWarpsPerBlock = 4;
 // double-precision set-up arithmetic per thread: GB300's FP64 pipe is narrow).
 
 // --------------------------------------------------------------------------
-// gather the charges into tree order
-// (blockIdx.y = RHS; qsm, when given, also receives the charges point-major:
-// qsm[k * rp + r], for the multi-RHS near field; qexp, when given, the biased
+// gather the charges into tree order (qexp, when given, receives the biased
 // exponent of the largest charge, for the double-precision near field's split)
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm,
-                           int64_t n, R *__restrict__ qs, R *__restrict__ qsm, int rp,
-                           int *__restrict__ qexp) {
+k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm, int64_t n,
+           R *__restrict__ qs, int *__restrict__ qexp) {
   pdl_wait();  // launched as a dependent of the tree build's last kernel
   pdl_trigger();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -76,88 +73,100 @@ k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm,
     }
   }
   if (k >= n) return;
-  const int r = blockIdx.y;
-  const double qd = q[(size_t)r * n + perm[k]];
-  R v;
+  const double qd = q[perm[k]];
   if constexpr (sizeof(R) == 4)
-    v = fs_round(qd);  // the rounding by integer operations (no FP64 conversion)
+    qs[k] = fs_round(qd);  // the rounding by integer operations (no FP64 conversion)
   else
-    v = qd;
-  qs[(size_t)r * n + k] = v;
-  if (qsm) qsm[(size_t)k * rp + r] = v;
+    qs[k] = qd;
 }
 
-// point position relative to its leaf centre, in units of the leaf side
-template <typename R>
-struct LeafPoints;
-
-template <>
-struct LeafPoints<double> {
-  const double *xs, *ys;
-  double x0;
-  __device__ __forceinline__ void rel(int64_t k, double cx, double cy, double &rx,
-                                      double &ry) const {
-    rx = xs[k] - cx;
-    ry = ys[k] - cy;
+// the same for nr charge vectors of a multi-RHS evaluation: qs[r n + k] and the
+// point-major copy qsm[k rp + r].  A warp takes 32 points, a vector at a time,
+// and turns them around in shared memory, so that both copies are written in
+// whole rows (one thread per value wrote qsm 4 bytes a sector: 360 us for 64
+// vectors of 500000).
+constexpr int kGmWarps = 4, kGmR = 32;  // vectors per block
+__global__ void __launch_bounds__(32 * kGmWarps)
+k_gather_multi(const double *__restrict__ q, const int64_t *__restrict__ perm, int64_t n, int nr,
+               float *__restrict__ qs, float *__restrict__ qsm, int rp) {
+  pdl_wait();  // launched as a dependent of the tree build's last kernel
+  pdl_trigger();
+  __shared__ float tile[32][kGmR + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t k0 = (int64_t)blockIdx.x * 32, k = k0 + lane;
+  const int r0 = blockIdx.y * kGmR;
+  const int64_t o = k < n ? perm[k] : 0;
+#pragma unroll
+  for (int j = warp; j < kGmR; j += kGmWarps) {
+    const int r = r0 + j;
+    float v = 0.0f;
+    if (r < nr && k < n) {
+      v = fs_round(q[(size_t)r * n + o]);
+      qs[(size_t)r * n + k] = v;
+    }
+    tile[lane][j] = v;
   }
-};
-template <>
-struct LeafPoints<float> {
-  const float2 *loc;
-  __device__ __forceinline__ void rel(int64_t k, double, double, float &rx, float &ry) const {
-    float2 v = loc[k];
-    rx = v.x;
-    ry = v.y;
-  }
-};
+  __syncthreads();
+  if (r0 + lane < rp)
+    for (int j = warp; j < 32; j += kGmWarps)
+      if (k0 + j < n) qsm[(size_t)(k0 + j) * rp + r0 + lane] = tile[j][lane];
+}
 
 // --------------------------------------------------------------------------
-// P2M (S2M, Eq. MEcoefficients up to the phase and conjugation, see tables.cu):
-// M_n = sum_{j in leaf} Q_j ((z_j - z_c)/d)^n.  One warp per leaf; lanes take
-// 32 points at a time, write q w^n into a shared buffer, then lanes sum the
-// buffer column by column.
-template <typename R>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-k_p2m(LeafPoints<R> pts, const R *__restrict__ qs, const int *__restrict__ leaf_start, int H,
-      const DevGeom *__restrict__ dg, int p, cpx<R> *__restrict__ M) {
-  const double x0 = dg->x0, side = dg->side;
+// Double-precision P2M (S2M, Eq. MEcoefficients up to the phase and
+// conjugation, see tables.cu): M_n = sum_{j in leaf} Q_j ((z_j - z_c)/d)^n.  A
+// block takes nlb consecutive leaves, whose points are one range: 128 points at
+// a time, a thread each, write q w^n into shared memory, then a thread per
+// (leaf, n) sums its leaf's column.  Bound by the FP64 pipe: four instructions a
+// point and order for the powers on full warps, two for the sums (a warp per
+// leaf of 15 points, 13 lanes summing, took 415 us at 1e6 points, p = 12).
+constexpr int kP2mThreads = 128, kP2mItems = 6;  // items a thread: 16 leaves x 41 orders / 128
+__global__ void __launch_bounds__(kP2mThreads)
+k_p2m64(const double *__restrict__ xs, const double *__restrict__ ys,
+        const double *__restrict__ qs, const int *__restrict__ leaf_start, int H, int nlb,
+        const DevGeom *__restrict__ dg, int p, cd *__restrict__ M) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  int P1 = p + 1;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  cpx<R> *buf = reinterpret_cast<cpx<R> *>(smem_raw) + (size_t)warp * P1 * 33;
-  int leaf = blockIdx.x * kWarpsPerBlock + warp;
-  int nleaf = 1 << (2 * H);
-  if (leaf >= nleaf) return;
-  double d = side / (double)(1 << H);
-  double cx = x0 + (box_ix(leaf) + 0.5) * d, cy = (box_iy(leaf) + 0.5) * d;
-  R invd = (R)(1.0 / d);
-  int b0 = leaf_start[leaf], b1 = leaf_start[leaf + 1];
-  cpx<R> acc0 = mk<R>(0, 0), acc1 = mk<R>(0, 0);
-  for (int base = b0; base < b1; base += 32) {
-    int k = base + lane;
-    int cnt = min(32, b1 - base);
-    if (k < b1) {
-      R rx, ry;
-      pts.rel(k, cx, cy, rx, ry);
-      cpx<R> w = mk<R>(rx * invd, ry * invd);
-      cpx<R> t = mk<R>(qs[k], 0);
+  cd *buf = reinterpret_cast<cd *>(smem_raw);  // [P1][129]
+  __shared__ int ls[17];
+  const int P1 = p + 1, L0 = blockIdx.x * nlb;
+  if (threadIdx.x <= nlb) ls[threadIdx.x] = leaf_start[L0 + threadIdx.x];
+  __syncthreads();
+  const double d = dg->side / (double)(1 << H), invd = 1.0 / d;
+  const int t0 = ls[0], t1 = ls[nlb], nit = nlb * P1;
+  cd acc[kP2mItems];
+#pragma unroll
+  for (int c = 0; c < kP2mItems; ++c) acc[c] = mk(0.0, 0.0);
+  for (int base = t0; base < t1; base += kP2mThreads) {
+    const int k = base + (int)threadIdx.x;
+    if (k < t1) {
+      int li = 0;  // the point's leaf: the last one whose start is <= k
+      for (int step = 8; step > 0; step >>= 1)
+        if (li + step < nlb && ls[li + step] <= k) li += step;
+      const double2 c = leaf_centre_at(dg->x0, d, box_ix(L0 + li), box_iy(L0 + li));
+      const cd w = mk((xs[k] - c.x) * invd, (ys[k] - c.y) * invd);
+      cd t = mk(qs[k], 0.0);
       for (int n = 0; n < P1; ++n) {
-        buf[n * 33 + lane] = t;
+        buf[n * 129 + threadIdx.x] = t;
         t = t * w;
       }
     }
-    __syncwarp();
-    for (int n = lane; n < P1; n += 32) {
-      cpx<R> s = mk<R>(0, 0);
-      for (int j = 0; j < cnt; ++j) s = s + buf[n * 33 + j];
-      if (n == lane) acc0 = acc0 + s;
-      else acc1 = acc1 + s;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kP2mItems; ++c) {
+      const int e = (int)threadIdx.x + c * kP2mThreads;
+      if (e < nit) {
+        const int leaf = e / P1, n = e - leaf * P1;
+        const int a = max(ls[leaf], base) - base, b = min(ls[leaf + 1], base + kP2mThreads) - base;
+        for (int i = a; i < b; ++i) acc[c] = acc[c] + buf[n * 129 + i];
+      }
     }
-    __syncwarp();
+    __syncthreads();
   }
-  cpx<R> *out = M + (size_t)(level_offset(H) + leaf) * P1;
-  if (lane < P1) out[lane] = acc0;
-  if (lane + 32 < P1) out[lane + 32] = acc1;
+#pragma unroll
+  for (int c = 0; c < kP2mItems; ++c) {
+    const int e = (int)threadIdx.x + c * kP2mThreads;
+    if (e < nit) M[(size_t)(level_offset(H) + L0) * P1 + e] = acc[c];
+  }
 }
 
 // --------------------------------------------------------------------------
@@ -178,22 +187,24 @@ __device__ __forceinline__ cpx<R> cpow_int(cpx<R> w, int n) {
 
 constexpr int kS2mGroup = 8;  // orders per thread of the single-precision S2M (a power of 2)
 
-// Single-precision S2M over a tile of kS2mLeaves consecutive leaves per block.
-// The tile's points are contiguous in tree order, so the block first copies
-// their leaf-frame positions and charges into shared memory with coalesced
-// loads (a per-thread loop over global memory would wait on one load per
-// point); a tile of more than kS2mCap points reads them from global memory
-// instead.  Each thread then takes items (leaf, group of kS2mGroup = G
-// consecutive orders n0 .. n0+G-1): w^n0 = (w^G)^(n0/G) from log2 G
-// squarings, then one product per further n.  The sums are compensated (Kahan): the moments of a
-// leaf are sums of up to hundreds of terms of both signs, and their rounding
-// error is inherited by every far-field coefficient built from them.
-constexpr int kS2mLeaves = 64, kS2mCap = 2048, kS2mThreads = 128;
+// Single-precision S2M over a tile of nlb consecutive leaves per block (64, or 16
+// or 4 where 64 would leave SMs idle).  The tile's points are contiguous in tree
+// order, so the block first copies their leaf-frame positions and charges into
+// shared memory with coalesced loads (a per-thread loop over global memory would
+// wait on one load per point); a tile of more than kS2mCap points reads them from
+// global memory instead.  S lanes take an item (leaf, group of kS2mGroup = G
+// consecutive orders n0 .. n0+G-1), each every S-th point of the leaf: w^n0 =
+// (w^G)^(n0/G) from log2 G squarings, then one product per further n.  The sums
+// are compensated (Kahan), the lanes' sums added pairwise: the moments of a leaf
+// are sums of up to hundreds of terms of both signs, and their rounding error is
+// inherited by every far-field coefficient built from them.  (50021 points in
+// 1024 leaves with one lane an item: 16 blocks, 61 us.)
+constexpr int kS2mCap = 2048, kS2mThreads = 128;
 
 __global__ void __launch_bounds__(kS2mThreads)
 k_s2m_tile(const float2 *__restrict__ loc, const float *__restrict__ qs,
-           const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg, int p,
-           cf *__restrict__ M, RhsStride rs) {
+           const int *__restrict__ leaf_start, int H, int nlb, int S,
+           const DevGeom *__restrict__ dg, int p, cf *__restrict__ M, RhsStride rs) {
   constexpr int G = kS2mGroup;
   __shared__ float2 sp[kS2mCap];
   __shared__ float sq[kS2mCap];
@@ -202,7 +213,7 @@ k_s2m_tile(const float2 *__restrict__ loc, const float *__restrict__ qs,
   qs += blockIdx.y * rs.q;
   M += blockIdx.y * rs.m;
   const int nleaf = 1 << (2 * H);
-  const int L0 = blockIdx.x * kS2mLeaves, L1 = min(L0 + kS2mLeaves, nleaf);
+  const int L0 = blockIdx.x * nlb, L1 = min(L0 + nlb, nleaf);
   const int t0 = leaf_start[L0], t1 = leaf_start[L1];
   const bool staged = t1 - t0 <= kS2mCap;
   if (staged) {
@@ -213,15 +224,17 @@ k_s2m_tile(const float2 *__restrict__ loc, const float *__restrict__ qs,
   }
   __syncthreads();
   const float invd = dg->invd[H];
-  for (int it = threadIdx.x; it < (L1 - L0) * NB; it += blockDim.x) {
-    const int leaf = L0 + it / NB, nb = it % NB, n0 = G * nb;
-    const int b0 = leaf_start[leaf], b1 = leaf_start[leaf + 1];
+  const int nit = (L1 - L0) * NB, part = (int)threadIdx.x & (S - 1);
+  for (int it0 = 0; it0 < nit; it0 += kS2mThreads / S) {
+    const int it = it0 + (int)threadIdx.x / S;
+    const int leaf = L0 + min(it, nit - 1) / NB, nb = it % NB, n0 = G * nb;
+    const int b0 = leaf_start[leaf], b1 = it < nit ? leaf_start[leaf + 1] : b0;
     // the compensated sums of the real and imaginary parts as paired FP32
     // additions (the same roundings as the scalar form)
     f2p acc[G], cmp[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) acc[g] = cmp[g] = f2_pack(0.f, 0.f);
-    for (int j = b0; j < b1; ++j) {
+    for (int j = b0 + part; j < b1; j += S) {
       const float2 v = staged ? sp[j - t0] : loc[j];
       const float qj = staged ? sq[j - t0] : qs[j];
       const cf w = mk(v.x * invd, v.y * invd);
@@ -241,12 +254,15 @@ k_s2m_tile(const float2 *__restrict__ loc, const float *__restrict__ qs,
     }
     const size_t e0 = ((size_t)level_offset(H) + leaf) * P1;
 #pragma unroll
-    for (int g = 0; g < G; ++g)
-      if (n0 + g < P1) {
-        float ax, ay;
-        f2_unpack(acc[g], ax, ay);
-        M[e0 + n0 + g] = mk(ax, ay);
+    for (int g = 0; g < G; ++g) {
+      float ax, ay;
+      f2_unpack(acc[g], ax, ay);
+      for (int o = 1; o < S; o <<= 1) {
+        ax += __shfl_xor_sync(0xffffffffu, ax, o);
+        ay += __shfl_xor_sync(0xffffffffu, ay, o);
       }
+      if (part == 0 && it < nit && n0 + g < P1) M[e0 + n0 + g] = mk(ax, ay);
+    }
   }
 }
 
@@ -299,11 +315,11 @@ k_s2m_multi(const float2 *__restrict__ loc, const float *__restrict__ qsm, int r
 // Fused upward pass.  The tree below level l0 = H - k is split into subtrees
 // of 4^k leaves; one block per subtree takes the leaf moments (S2M kernel) and
 // merges them level by level up to l0 with the M2M shift (Eq. metome) in
-// shared memory.  When the levels above l0 are small (l0 <= kCoarseBig), the
-// block that finishes last (a counter in global memory) also runs them, l0 - 1
-// down to 1, so the upward pass needs no further launch; deeper trees run
-// them as separate launches.
-constexpr int kCoarseBig = 5;  // coarse levels with at least 4^5 boxes get a multi-block launch
+// shared memory.  When the levels above are small (l0 <= kCoarse), the block
+// that finishes last (a counter in global memory) also runs them, l0 - 1 down to 1, so the upward pass needs no
+// further launch; deeper trees launch each level down to kCoarse over many
+// blocks and the rest as one block.
+constexpr int kCoarse = 4;
 
 // a complex number read past L1 (written by another block of the same launch)
 __device__ __forceinline__ cf ldcg_c(const cf *p) {
@@ -366,17 +382,37 @@ __device__ __forceinline__ void m2m_levels_smem(cpx<R> *child, int nchild, int l
     cpx<R> *par = child + (size_t)((nchild + 3) >> 2) * GS;
     const int npar = nchild >> 2;
     const int64_t first = first_child >> (2 * (lc - l));
-    for (int e = threadIdx.x; e < npar * P1; e += blockDim.x) {
-      const int n = e / npar, b = e - n * npar;
-      cpx<R> acc = mk<R>(0, 0);
-      const cpx<R> *mg = child + (size_t)b * GS;  // the four children of parent b
+    if (npar >= 32) {
+      for (int e = threadIdx.x; e < npar * P1; e += blockDim.x) {
+        const int n = e / npar, b = e - n * npar;
+        cpx<R> acc = mk<R>(0, 0);
+        const cpx<R> *mg = child + (size_t)b * GS;  // the four children of parent b
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const cpx<R> *Tc = T + (size_t)c * P1 * P1 + (size_t)n * P1;
-        const cpx<R> *mc = mg + c * P1;
-        for (int m = 0; m <= n; ++m) cfma(acc, Tc[m], mc[m]);
+        for (int c = 0; c < 4; ++c) {
+          const cpx<R> *Tc = T + (size_t)c * P1 * P1 + (size_t)n * P1;
+          const cpx<R> *mc = mg + c * P1;
+          for (int m = 0; m <= n; ++m) cfma(acc, Tc[m], mc[m]);
+        }
+        par[m2m_slot<R>(b, n, P1)] = acc;
       }
-      par[m2m_slot<R>(b, n, P1)] = acc;
+    } else {
+      // few parents: a lane per child, a quarter of the chain
+      for (int e0 = 0; e0 < 4 * npar * P1; e0 += blockDim.x) {
+        const int e = e0 + (int)threadIdx.x, it = e >> 2, c = e & 3;
+        const int n = it / npar, b = it - n * npar;
+        cpx<R> acc = mk<R>(0, 0);
+        if (it < npar * P1) {
+          const cpx<R> *mc = child + (size_t)b * GS + c * P1;
+          const cpx<R> *Tc = T + (size_t)c * P1 * P1 + (size_t)n * P1;
+          for (int m = 0; m <= n; ++m) cfma(acc, Tc[m], mc[m]);
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+          acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+          acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+        }
+        if (c == 0 && it < npar * P1) par[m2m_slot<R>(b, n, P1)] = acc;
+      }
     }
     __syncthreads();
     const size_t o = (size_t)(level_offset(l) + first) * P1;
@@ -389,9 +425,37 @@ __device__ __forceinline__ void m2m_levels_smem(cpx<R> *child, int nchild, int l
   }
 }
 
+// Levels l0 - 1 .. 1 (l0 <= kCoarse) by one block, from the moments of level l0 in
+// global memory (read past L1: other blocks wrote them), `room` (64 or 256) boxes
+// at a time.  With room for all 256 of level 4 (64 KB at p = 16) the blocks of the
+// upward pass wait for the near field's to leave their SMs (0.50 -> 0.65 ms an
+// evaluation, 1e6 points, leaves of 61), so that is for trees whose near field is
+// short, or whose subtrees need that much anyway.
+template <typename R>
+__device__ __forceinline__ void m2m_top(cpx<R> *Ms, int l0, int room, int P1,
+                                        const cpx<R> *__restrict__ T, cpx<R> *__restrict__ M) {
+  const int nb0 = 1 << (2 * l0), chunk = nb0 < room ? nb0 : room;
+  for (int b0 = 0; b0 < nb0; b0 += chunk) {
+    for (int e = threadIdx.x; e < chunk * P1; e += blockDim.x) {
+      const int b = e / P1, m = e - b * P1;
+      Ms[m2m_slot<R>(b, m, P1)] = ldcg_c(M + (size_t)(level_offset(l0) + b0) * P1 + e);
+    }
+    __syncthreads();
+    m2m_levels_smem<R>(Ms, chunk, l0, nb0 > chunk ? l0 - 1 : 1, b0, P1, T, M);
+    __syncthreads();
+  }
+  if (nb0 == chunk) return;
+  for (int e = threadIdx.x; e < 64 * P1; e += blockDim.x) {  // level 3, just written
+    const int b = e / P1, m = e - b * P1;
+    Ms[m2m_slot<R>(b, m, P1)] = ldcg_c(M + (size_t)level_offset(3) * P1 + e);
+  }
+  __syncthreads();
+  m2m_levels_smem<R>(Ms, 64, 3, 1, 0, P1, T, M);
+}
+
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_upward(int H, int k, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restrict__ M,
+k_upward(int H, int k, int room, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restrict__ M,
          RhsStride rs, int *__restrict__ ctr) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int s_last;
@@ -411,9 +475,7 @@ k_upward(int H, int k, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restric
   __syncthreads();
   // M2M inside the subtree: level H-1 .. H-k
   m2m_levels_smem<R>(Ms, nl, H, H - k, first_leaf, P1, T, M);
-  // the coarse levels l0 - 1 .. 1, by the last block to finish, from the
-  // 4^l0 moments of level l0 staged in shared memory (l0 <= k: they fit where
-  // the subtree was)
+  // the coarse levels l0 - 1 .. 1, by the last block to finish
   const int l0 = H - k;
   if (!ctr || l0 <= 1) return;
   __threadfence();
@@ -422,31 +484,26 @@ k_upward(int H, int k, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restric
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const int nb0 = 1 << (2 * l0);
-  for (int e = threadIdx.x; e < nb0 * P1; e += blockDim.x) {
-    const int b = e / P1, m = e - b * P1;
-    Ms[m2m_slot<R>(b, m, P1)] = ldcg_c(M + (size_t)level_offset(l0) * P1 + e);
-  }
-  __syncthreads();
-  m2m_levels_smem<R>(Ms, nb0, l0, 1, 0, P1, T, M);
+  m2m_top<R>(Ms, l0, room, P1, T, M);
   if (threadIdx.x == 0) ctr[blockIdx.y] = 0;  // ready for the next launch
 }
 
-// M2M for the small coarse levels lhi .. 1, one block, level by level
+// M2M for the small coarse levels l0 - 1 .. 1 in one block, staged in shared
+// memory (read from global memory, one dependent round trip a term, levels
+// 3 .. 1 took 68 us at p = 16)
 template <typename R>
-__global__ void __launch_bounds__(1024)
-k_m2m_coarse(int lhi, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restrict__ M,
+__global__ void __launch_bounds__(512)
+k_m2m_coarse(int l0, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restrict__ M,
              RhsStride rs) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   const int P1 = p + 1;
   M += blockIdx.y * rs.m;
-  for (int l = lhi; l >= 1; --l) {
-    const int nb = 1 << (2 * l);
-    for (int e = threadIdx.x; e < nb * P1; e += blockDim.x) m2m_item<R>(l, e, P1, Tm2m, M);
-    __syncthreads();
-  }
+  cpx<R> *T = reinterpret_cast<cpx<R> *>(smem_raw);
+  for (int e = threadIdx.x; e < 4 * P1 * P1; e += blockDim.x) T[e] = Tm2m[e];
+  m2m_top<R>(T + 4 * P1 * P1, l0, 64, P1, T, M);
 }
 
-// the same for one level with many boxes, one thread per (box, n) over many blocks
+// M2M of one level with many boxes, one thread per (box, n) over many blocks
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_m2m_level(int l, int p, const cpx<R> *__restrict__ Tm2m, cpx<R> *__restrict__ M, RhsStride rs) {
@@ -672,12 +729,7 @@ k_downward(int H, int k, int p, const cpx<R> *__restrict__ Tl2l, cpx<R> *__restr
       const double2 c = leaf_centre_at(ev.dg->x0, d, ix, iy);
       const cd w = mk((ev.xs[i] - c.x) * invd, (ev.ys[i] - c.y) * invd), wb = conj(w);
       cd va = Al[p], da = mk(0.0, 0.0), vb = Bl[p], db = mk(0.0, 0.0);
-      for (int n = p - 1; n >= 0; --n) {
-        da = da * w + va;
-        va = va * w + Al[n];
-        db = db * wb + vb;
-        vb = vb * wb + Bl[n];
-      }
+      for (int n = p - 1; n >= 0; --n) horner4(va, da, vb, db, w, wb, Al[n], Bl[n]);
       const double lf = ev.near64[i], fx = ev.near64[ev.n + i], fy = ev.near64[2 * ev.n + i];
       cd u = va + vb, gx = invd * (da + db), gy = invd * (mul_i(da) - mul_i(db));
       u.x = fma(-0.5 * i2pi, lf, u.x);
@@ -720,12 +772,7 @@ k_downward(int H, int k, int p, const cpx<R> *__restrict__ Tl2l, cpx<R> *__restr
       const float4 nv = cu.near;
       const cf w = mk(me.x * invd, me.y * invd), wb = conj(w);
       cf va = Al[p], da = mk(0.f, 0.f), vb = Bl[p], db = mk(0.f, 0.f);
-      for (int n = p - 1; n >= 0; --n) {
-        da = da * w + va;
-        va = va * w + Al[n];
-        db = db * wb + vb;
-        vb = vb * wb + Bl[n];
-      }
+      for (int n = p - 1; n >= 0; --n) horner4(va, da, vb, db, w, wb, Al[n], Bl[n]);
       const float ur_ = va.x + vb.x - nv.x * c4;
       const float ui_ = va.y + vb.y;
       const cf gxo = invd * (da + db) + mk(-nv.y * i2pi, 0.f);
@@ -758,6 +805,7 @@ size_t upward_smem(int p, int k) {
   for (int j = 0; j <= k; ++j) ng += (size_t(1) << (2 * j) >> 2) > 0 ? (size_t(1) << (2 * j)) >> 2 : 1;
   return sizeof(cpx<R>) * (4 * (size_t)P1 * P1 + ng * m2m_group_stride<R>(P1));
 }
+size_t p2m64_smem(int p) { return sizeof(cd) * 129 * (size_t)(p + 1); }
 template <typename R>
 size_t downward_smem(int p, int k, bool eval) {
   const size_t P1 = p + 1;
@@ -854,22 +902,20 @@ k_m2l_free(int l, int p, const DevGeom *__restrict__ dg, const cpx<R> *__restric
 
 // --------------------------------------------------------------------------
 // The patch form of the free-space M2L (m2l_patch.cuh) is instantiated for
-// every order in two translation units; this dispatches on p.
-template <typename R>
-bool launch_m2l_patch(int p, int H, int lmin, int lmax, const DevGeom *dg, const cpx<R> *Tpad,
-                      const cd *logt, const cpx<R> *M, cpx<R> *A, cpx<R> *B, int *status,
-                      cudaStream_t st, int nr, RhsStride rs, const int *leaf_start,
-                      int skip_empty) {
-  if constexpr (sizeof(R) == 8) {
-    return m2l_patch_launch_64(p, H, lmin, lmax, dg, Tpad, logt, M, A, B, status, st, nr, rs,
-                               leaf_start, skip_empty);
-  } else {
-    if (p <= kPatchSplitP)
-      return m2l_patch_launch_lo(p, H, lmin, lmax, dg, Tpad, logt, M, A, B, status, st, nr, rs,
-                                 leaf_start, skip_empty);
-    return m2l_patch_launch_hi(p, H, lmin, lmax, dg, Tpad, logt, M, A, B, status, st, nr, rs,
-                               leaf_start, skip_empty);
-  }
+// every order in several translation units; this dispatches on p.
+inline bool launch_m2l_patch(HP_PATCH_ARGS(cf)) {
+  if (!Tpad || p < 2 || p > HPFMM_MAX_P) return false;
+  auto *go = p <= kPatchOrders[0] ? m2l_patch_launch_f0
+                                  : (p <= kPatchOrders[1] ? m2l_patch_launch_f1 : m2l_patch_launch_f2);
+  return go(p, H, lmin, lmax, dg, Tpad, logt, M, A, B, status, st, nr, rs, leaf_start,
+            skip_empty);
+}
+inline bool launch_m2l_patch(HP_PATCH_ARGS(cd)) {
+  if (!Tpad || p < 2 || p > HPFMM_MAX_P) return false;
+  auto *go = p <= kPatchOrders[0] ? m2l_patch_launch_d0
+                                  : (p <= kPatchOrders[1] ? m2l_patch_launch_d1 : m2l_patch_launch_d2);
+  return go(p, H, lmin, lmax, dg, Tpad, logt, M, A, B, status, st, nr, rs, leaf_start,
+            skip_empty);
 }
 
 // --------------------------------------------------------------------------
@@ -1097,7 +1143,8 @@ bool launch_m2l_tc(int p, int H, const DevGeom *dg, const float *Btab, const cd 
 // All-levels form of the mirror M2L: one block of 4 warps per target box of
 // rows 0 and 1 of every level 1..H; the warps split the (at most 12) sources
 // of the mirror list, lanes run over the output index, and the four partial
-// sums are reduced in shared memory.  Without Amir / Bmir, level 1
+// sums are reduced in shared memory; the matrices are stored with the output
+// order last, so that a warp reads a row of them at once.  Without Amir / Bmir, level 1
 // initialises A and B and deeper levels add to the free-space result; with
 // them, the results go there instead (box t of the launch at t (p+1), see
 // mirror_slot), so that this kernel need not wait for the free-space M2L.
@@ -1148,9 +1195,9 @@ k_m2l_mirror_all(int H, int p, const DevGeom *__restrict__ dg, const cpx<R> *__r
         cpx<R> sL = mk<R>(0, 0), sC = mk<R>(0, 0), sD = mk<R>(0, 0);
         for (int k = 0; k < P1; ++k) {
           cpx<R> mv = ms[k], mc = conj(mv);
-          cfma(sL, Ti[n * P1 + k], mc);
-          cfma(sC, Tp[n * P1 + k], mc);
-          cfma(sD, Tm[n * P1 + k], mv);
+          cfma(sL, Ti[k * P1 + n], mc);
+          cfma(sC, Tp[k * P1 + n], mc);
+          cfma(sD, Tm[k * P1 + n], mv);
         }
         if (n == 0) sL.x += ms[0].x * ((R)logimg[cls].x + logd);  // M_0 ln|t d|
         aL[r] = aL[r] + sL;
@@ -1210,12 +1257,6 @@ struct SrcPt32 { float x, y, q, pad; };
 // skips coincident positions (r^2 = 0), i.e. the j = i pair.
 constexpr int kEvWarps = 8;
 
-__device__ __forceinline__ void mirror_batch(const float4 *buf, int cnt, int g, int ng, float mx,
-                                             float my, cf kap, const KappaLog &K, float tau,
-                                             NearAcc &a) {
-  for (int k = g; k < cnt; k += ng) mirror_pair(buf[k], mx, my, kap, K, tau, a);
-}
-
 __device__ __forceinline__ float xsum(float v, int from) {
 #pragma unroll 1
   for (int o = from; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1223,27 +1264,34 @@ __device__ __forceinline__ float xsum(float v, int from) {
 }
 
 // tile geometry of the single-precision leaf kernel
-constexpr int kTl = 4;             // target leaves per tile side
+constexpr int kTl = 4;             // target leaves per tile side, at most
 constexpr int kTlP = kTl + 2;      // patch leaves per side
-constexpr int kTlCap = 2560;       // staged points per block
+constexpr int kTlCap = 1280;       // staged points per block
 constexpr int kLsBytes = 80;       // tile leaf starts (kTl^2 + 1 ints), 16-byte padded
 
 // Single-precision free-space near field (the j != i sum of Eq. 1.2 over the
 // 3 x 3 leaf neighbourhood of each target), one target per lane.  A block
-// takes a 4 x 4 tile of leaves -- 16 consecutive Morton leaves, so its
-// targets are one contiguous range of the sorted points -- and stages the
-// 6 x 6 leaves around it in shared memory, row by row: each point's position
-// in the frame of the tile's first leaf as a float pair (hi, lo), converted
-// once from its leaf frame by an exact two-sum with the leaf's offset (a
-// multiple of the leaf side, itself split into hi + lo), and its charge.  A
-// row of a target's neighbourhood is then one contiguous range of the staged
-// points, and a pair difference (x_i - x_j) = (hi_i - hi_j) + (lo_i - lo_j)
-// is exact up to its one rounding: without the lo parts the float frames
+// takes a tile of tl x tl leaves (4 x 4, or 2 x 2 for full leaves) -- consecutive
+// Morton leaves, so its targets are one contiguous range of the sorted points --
+// and stages the leaves of the tile and around it in shared memory, row by row:
+// each point's position in the frame of the tile's first leaf as a float pair
+// (hi, lo), converted once from its leaf frame by an exact two-sum with the
+// leaf's offset (a multiple of the leaf side, itself split into hi + lo), and
+// its charge.  A row of a target's neighbourhood is then one contiguous range of
+// the staged points, and a pair difference (x_i - x_j) = (hi_i - hi_j) + (lo_i -
+// lo_j) is exact up to its one rounding: without the lo parts the float frames
 // would cost close pairs their relative precision (an absolute error of
 // about 2^-25 d in every difference).  The target's own point is skipped by
 // index.  Lanes of one warp may belong to two or three leaves: they run the
-// same loops with their own bounds.  Patches larger than the buffer read
-// from global memory, leaf by leaf in leaf frames.
+// same loops with their own bounds.  A 4 x 4 tile whose patch exceeds the buffer
+// is taken as four 2 x 2 tiles; a 2 x 2 tile's patch that still does reads from
+// global memory, leaf by leaf in leaf frames.
+//
+// The buffer (26 KB) is kept small because the far-field kernels run beside
+// this one and need shared memory of their own on the same SMs: with 61 KB (one
+// 4 x 4 tile of leaves of 71 points) they waited for this kernel's blocks to
+// finish.  For the same reason full leaves take 2 x 2 tiles, whose blocks end
+// after a quarter of the time.
 // the free-space pairs of one target (tile-frame position mh + ml, as (x, y)
 // pairs) with the staged sources lo .. hi - 1: lf += q log2 r^2 and
 // g += q (dx, dy) / r^2, the differences formed as (hi - hi) + (lo - lo)
@@ -1307,16 +1355,16 @@ __device__ __forceinline__ void add_hilo(float h, float l, float oh, float ol, f
   sl = (l + ol) + e;
 }
 
-__global__ void __launch_bounds__(kEvWarps * 32, 4)
-k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
-         const double *__restrict__ q, const int64_t *__restrict__ perm,
-         const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg,
-         float4 *__restrict__ near) {
-  // launched as a dependent of the tree build's last kernel; the charges are
-  // read in the caller's order through perm and rounded as the charge gather
-  // rounds them (bit-identical to the gathered copy), so that the gather runs
-  // beside this kernel instead of before it
-  pdl_wait();
+// one tile of TL x TL leaves (fewer on a smaller tree) from leaf (tx0, ty0); false
+// when its patch exceeds the buffer and the caller takes it in quarters
+template <int TL>
+__device__ __forceinline__ bool near_tile(int tx0, int ty0, int nx, float d, float dlo,
+                                          const float2 *__restrict__ loc,
+                                          const float2 *__restrict__ loclo,
+                                          const double *__restrict__ q,
+                                          const int64_t *__restrict__ perm,
+                                          const int *__restrict__ leaf_start,
+                                          float4 *__restrict__ near) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   int *ls = reinterpret_cast<int *>(smem_raw);         // [kTl^2 + 1] tile leaf starts
   float4 *src = reinterpret_cast<float4 *>(smem_raw + kLsBytes);  // [kTlCap] (hi, lo)
@@ -1324,19 +1372,16 @@ k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
   int *pst = reinterpret_cast<int *>(srcq + kTlCap);   // [kTlP^2 + 1]
   int *pbeg = pst + kTlP * kTlP + 1;                   // [kTlP^2]
   __shared__ float offh[kTlP], offl[kTlP];             // (c - 1) d as hi + lo, c = 0..5
-  const float d = dg->d[H], dlo = dg->dlo[H];
+  constexpr int ps = TL + 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nx = 1 << H;
-  const int tps = nx >= kTl ? nx / kTl : 1;
-  const int tx0 = (blockIdx.x % tps) * kTl, ty0 = (blockIdx.x / tps) * kTl;
-  const int side = nx < kTl ? nx : kTl, nlt = side * side;
+  const int side = nx < TL ? nx : TL, nlt = side * side;
   const uint64_t L0 = box_morton(tx0, ty0);
   if (warp == 0) {
     int c0 = 0, c1 = 0;
     for (int h = 0; h < 2; ++h) {
       const int pi = lane + 32 * h;
-      if (pi < kTlP * kTlP) {
-        const int lx = tx0 - 1 + pi % kTlP, ly = ty0 - 1 + pi / kTlP;
+      if (pi < ps * ps) {
+        const int lx = tx0 - 1 + pi % ps, ly = ty0 - 1 + pi / ps;
         int b0 = 0, cnt = 0;
         if (lx >= 0 && ly >= 0 && lx < nx && ly < nx) {
           const uint64_t lf = box_morton(lx, ly);
@@ -1353,9 +1398,9 @@ k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
       if (lane >= o) { i0 += a0; i1 += a1; }
     }
     const int tot0 = __shfl_sync(0xffffffffu, i0, 31);
+    // (entries past ps^2 hold the total)
     pst[lane] = i0 - c0;
-    if (lane + 32 < kTlP * kTlP) pst[lane + 32] = tot0 + i1 - c1;
-    if (lane == kTlP * kTlP - 32 - 1) pst[kTlP * kTlP] = tot0 + i1;
+    if (lane <= kTlP * kTlP - 32) pst[lane + 32] = tot0 + i1 - c1;
   } else if (warp == 1 && lane <= nlt) {
     ls[lane] = leaf_start[L0 + lane];
   } else if (warp == 2 && lane < kTlP) {
@@ -1366,12 +1411,13 @@ k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
     offl[lane] = (float)(o - (double)oh);
   }
   __syncthreads();
-  const bool staged = pst[kTlP * kTlP] <= kTlCap;
+  const bool staged = pst[ps * ps] <= kTlCap;
+  if (!staged && TL > 2) return false;  // (the same for the whole block)
   if (staged) {
-    for (int pi = warp; pi < kTlP * kTlP; pi += kEvWarps) {
+    for (int pi = warp; pi < ps * ps; pi += kEvWarps) {
       const int b0 = pbeg[pi], cnt = pst[pi + 1] - pst[pi], o = pst[pi];
-      const float ohx = offh[pi % kTlP], olx = offl[pi % kTlP];
-      const float ohy = offh[pi / kTlP], oly = offl[pi / kTlP];
+      const float ohx = offh[pi % ps], olx = offl[pi % ps];
+      const float ohy = offh[pi / ps], oly = offl[pi / ps];
       for (int j = lane; j < cnt; j += 32) {
         const float2 v = loc[b0 + j], w = loclo[b0 + j];
         float hx, lx, hy, ly;
@@ -1396,14 +1442,14 @@ k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
     const int px = ix - tx0 + 1, py = iy - ty0 + 1;
     float lf = 0.f, gx = 0.f, gy = 0.f;
     if (staged) {
-      const int kself = pst[py * kTlP + px] + (i - ls[li]);
+      const int kself = pst[py * ps + px] + (i - ls[li]);
       float4 me = make_float4(0.f, 0.f, 0.f, 0.f);
       if (act) me = src[kself];
       const f2p mh = f2_pack(me.x, me.y), ml = f2_pack(me.z, me.w);
       f2p g = f2_pack(0.f, 0.f);
 #pragma unroll 1
       for (int r = -1; r <= 1; ++r) {
-        const int pi = (py + r) * kTlP + px;
+        const int pi = (py + r) * ps + px;
         const int lo = pst[pi - 1];
         const int hi = act ? pst[pi + 2] : lo;
         if (r == 0) {
@@ -1440,6 +1486,31 @@ k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
       }
     }
     if (act) near[i] = make_float4(lf, gx, gy, 0.f);
+  }
+  return true;
+}
+
+template <int TL>
+__global__ void __launch_bounds__(kEvWarps * 32, 4)
+k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
+         const double *__restrict__ q, const int64_t *__restrict__ perm,
+         const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg,
+         float4 *__restrict__ near) {
+  // launched as a dependent of the tree build's last kernel; the charges are
+  // read in the caller's order through perm and rounded as the charge gather
+  // rounds them (bit-identical to the gathered copy), so that the gather runs
+  // beside this kernel instead of before it
+  pdl_wait();
+  const float d = dg->d[H], dlo = dg->dlo[H];
+  const int nx = 1 << H, tps = nx >= TL ? nx / TL : 1;
+  const int tx0 = (blockIdx.x % tps) * TL, ty0 = (blockIdx.x / tps) * TL;
+  if (near_tile<TL>(tx0, ty0, nx, d, dlo, loc, loclo, q, perm, leaf_start, near)) return;
+  if constexpr (TL > 2) {
+    for (int s = 0; s < 4; ++s) {
+      const int x = tx0 + 2 * (s & 1), y = ty0 + 2 * (s >> 1);
+      __syncthreads();  // the staged points are replaced
+      if (x < nx && y < nx) near_tile<2>(x, y, nx, d, dlo, loc, loclo, q, perm, leaf_start, near);
+    }
   }
 }
 constexpr size_t kTpSmem = kLsBytes + (sizeof(float4) + sizeof(float)) * kTlCap +
@@ -1630,12 +1701,7 @@ k_eval32m(const float2 *__restrict__ loc, const float *__restrict__ qsm, int rp,
       if (r >= nr) break;
       const cf *Al = A + r * rs.m + le, *Bl = B + r * rs.m + le;
       cf va = Al[p], da = mk(0.f, 0.f), vb = Bl[p], db = mk(0.f, 0.f);
-      for (int n = p - 1; n >= 0; --n) {
-        da = da * w + va;
-        va = va * w + Al[n];
-        db = db * wb + vb;
-        vb = vb * wb + Bl[n];
-      }
+      for (int n = p - 1; n >= 0; --n) horner4(va, da, vb, db, w, wb, Al[n], Bl[n]);
       const float ur_ = va.x + vb.x - a.lf[c] * c4;
       const float ui_ = va.y + vb.y;
       const cf gxo = invd * (da + db) + mk(-a.gx[c] * i2pi, 0.f);
@@ -1702,12 +1768,7 @@ k_eval_targets(const double *__restrict__ xt, const double *__restrict__ yt, int
     const cpx<R> *Bl = B + (size_t)(level_offset(H) + leaf) * P1;
     const cpx<R> w = mk((R)lx * rinvd, (R)ly * rinvd), wb = conj(w);
     cpx<R> va = Al[p], da = mk<R>(0, 0), vb = Bl[p], db = mk<R>(0, 0);
-    for (int n = p - 1; n >= 0; --n) {
-      da = da * w + va;
-      va = va * w + Al[n];
-      db = db * wb + vb;
-      vb = vb * wb + Bl[n];
-    }
+    for (int n = p - 1; n >= 0; --n) horner4(va, da, vb, db, w, wb, Al[n], Bl[n]);
     auto c64 = [](cpx<R> z) { return mk((double)z.x, (double)z.y); };
     u = c64(va + vb);
     gx = (1.0 / d) * c64(da + db);
@@ -1818,103 +1879,134 @@ k_eval_targets(const double *__restrict__ xt, const double *__restrict__ yt, int
   }
 }
 
-// Image and reaction near field of the bottom-row leaves (single precision
-// with the double routine for |P| > 1 and, in MIXED mode, below tau), added
-// to the outputs written by the leaf kernel.  One block per bottom-row leaf: the
-// sources of the three bottom-row neighbours are staged in shared memory,
-// lanes take 32 targets at a time and the 8 warps split the sources; the
-// partial sums are reduced in shared memory.
-constexpr int kMirSrc = 512;
-constexpr int kMirSplit = 8;  // blocks per bottom-row leaf
-__global__ void __launch_bounds__(kEvWarps * 32)
+// Sources of a bottom-row leaf's image and reaction pairs: the up to three
+// bottom-row leaves beside it, as one range of entries.
+struct MirrorRange {
+  int s[3], c01, c012, c0;
+  __device__ __forceinline__ void set(const int *__restrict__ leaf_start, int ix, int nx) {
+    int cnt[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int mx = ix - 1 + k;
+      s[k] = cnt[k] = 0;
+      if (mx >= 0 && mx < nx) {
+        const uint64_t sl = box_morton(mx, 0);
+        s[k] = leaf_start[sl];
+        cnt[k] = leaf_start[sl + 1] - s[k];
+      }
+    }
+    c0 = cnt[0];
+    c01 = c0 + cnt[1];
+    c012 = c01 + cnt[2];
+  }
+  // entry e: its leaf (0, 1, 2: left, same, right) and its point
+  __device__ __forceinline__ int point(int e, int &k) const {
+    k = e < c0 ? 0 : (e < c01 ? 1 : 2);
+    return e < c0 ? s[0] + e : (e < c01 ? s[1] + e - c0 : s[2] + e - c01);
+  }
+};
+
+// Image and reaction near field of the bottom-row leaves (single precision,
+// the double routine for |P| > 1 and, in MIXED mode, below tau).  16 lanes a
+// target stride over its sources; grid (leaf, 1, split), the targets of a leaf
+// spread over the blocks' groups.  The pairs are few but long, so what counts is
+// that they spread: with 32 targets a warp and the sources split over 8 warps,
+// leaves of 61 points kept 256 of 1024 blocks busy and took 286 us.
+constexpr int kMirThreads = 128, kMirSplit = 8;
+__global__ void __launch_bounds__(kMirThreads, 6)
 k_mirror32(const float2 *__restrict__ loc, const float *__restrict__ yabs,
            const float *__restrict__ qs,
            const int64_t *__restrict__ perm, const int *__restrict__ leaf_start, int H,
            const DevGeom *__restrict__ dg, KappaLog K, float tau, double *__restrict__ pot,
-           double *__restrict__ grad, RhsStride rs, int assign) {
-  const float d = dg->d[H];
-  qs += blockIdx.y * rs.q;
-  pot += blockIdx.y * rs.out;
-  if (grad) grad += blockIdx.y * 2 * rs.out;
-  __shared__ float4 src[kMirSrc];
-  __shared__ float red[kEvWarps][9][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nx = 1 << H;
-  const int ix = blockIdx.x;  // leaf (ix, 0)
-  const cf kap = mk((float)K.kappa.x, (float)K.kappa.y);
+           double *__restrict__ grad) {
+  constexpr int G = 16;
+  const int ix = blockIdx.x, lane = threadIdx.x & (G - 1), grp = threadIdx.x / G;
+  const unsigned mask = 0xffffu << (threadIdx.x & 16);
   const uint64_t leaf = box_morton(ix, 0);
   const int b0 = leaf_start[leaf], b1 = leaf_start[leaf + 1];
-  // source ranges of the bottom-row neighbours
-  int s0[3], s1[3];
-  float ox[3];
-  int ns = 0;
-  for (int k = 0; k < 3; ++k) {
-    int mxx = ix - 1 + k;
-    s0[k] = s1[k] = 0;
-    ox[k] = (float)(mxx - ix) * d;
-    if (mxx >= 0 && mxx < nx) {
-      uint64_t sl = box_morton(mxx, 0);
-      s0[k] = leaf_start[sl];
-      s1[k] = leaf_start[sl + 1];
+  const int stride = kMirThreads / G * (int)gridDim.z;
+  int i = b0 + grp + kMirThreads / G * (int)blockIdx.z;
+  if (i >= b1) return;
+  const float d = dg->d[H];
+  const KappaF kf = kappa_f(K);
+  MirrorRange src;
+  src.set(leaf_start, ix, 1 << H);
+  for (; i < b1; i += stride) {
+    const float mx = loc[i].x, my = yabs[i];
+    MirrorAcc acc;
+    acc.clear();
+    for (int e = lane; e < src.c012; e += G) {
+      int k;
+      const int j = src.point(e, k);
+      const float sx = loc[j].x + (float)(k - 1) * d;
+      acc.add(qs[j], mirror_value(mx - sx, my + yabs[j], kf, K, tau));
     }
-    ns += s1[k] - s0[k];
+    acc.reduce<G>(mask);
+    if (lane == 0) acc.put(pot, grad, perm[i], true);
   }
-  const float c4 = (float)(0.69314718055994530942 / (4.0 * HP_PI));
-  const float i2pi = (float)(1.0 / HP_TWO_PI);
-  // target tiles of 32 are spread over gridDim.z blocks (leaves next to a
-  // cluster hold many points)
-  for (int tb = b0 + 32 * (int)blockIdx.z; tb < b1; tb += 32 * (int)gridDim.z) {
-    const int i = tb + lane;
-    const bool act = i < b1;
-    const float2 me = act ? make_float2(loc[i].x, yabs[i]) : make_float2(0.f, 0.f);
-    NearAcc acc;
-    acc.lf = acc.gx = acc.gy = acc.li = acc.gix = acc.giy = 0.f;
-    acc.ur = acc.grx = acc.gry = mk(0.f, 0.f);
-    for (int base = 0; base < ns; base += kMirSrc) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < kMirSrc && base + e < ns; e += blockDim.x) {
-        int r = base + e, k = 0;
-        while (r >= s1[k] - s0[k]) { r -= s1[k] - s0[k]; ++k; }
-        const int js = s0[k] + r;
-        const float2 v = loc[js];
-        src[e] = make_float4(v.x + ox[k], yabs[js], qs[js], 0.f);
+}
+
+// The same for many charge vectors (added to the outputs of the leaf kernel): a
+// warp takes a target, its lanes 32 sources' pair values at a time, which go
+// through shared memory to lanes that take one charge vector each (RB = 32 or 64
+// in all; charges point-major, qsm[k * rp + r], one coalesced row a source).  A
+// pair's 130 instructions serve all vectors, which then take six products each.
+constexpr int kMirmWarps = 4;
+template <int RB>
+__global__ void __launch_bounds__(32 * kMirmWarps)
+k_mirror32m(const float2 *__restrict__ loc, const float *__restrict__ yabs,
+            const float *__restrict__ qsm, int rp, int nr, const int64_t *__restrict__ perm,
+            const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg, KappaLog K,
+            float tau, double *__restrict__ pot, double *__restrict__ grad, RhsStride rs) {
+  constexpr int NB = RB / 32;
+  __shared__ float4 sv[kMirmWarps][32];
+  __shared__ float2 sw[kMirmWarps][32];
+  __shared__ int sj[kMirmWarps][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ix = blockIdx.x;
+  const uint64_t leaf = box_morton(ix, 0);
+  const int b0 = leaf_start[leaf], b1 = leaf_start[leaf + 1];
+  const float d = dg->d[H];
+  const KappaF kf = kappa_f(K);
+  MirrorRange src;
+  src.set(leaf_start, ix, 1 << H);
+  for (int i = b0 + warp + kMirmWarps * (int)blockIdx.z; i < b1; i += kMirmWarps * (int)gridDim.z) {
+    const float mx = loc[i].x, my = yabs[i];
+    MirrorAcc acc[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) acc[b].clear();
+    for (int base = 0; base < src.c012; base += 32) {
+      const int cnt = min(32, src.c012 - base);
+      __syncwarp();
+      if (lane < cnt) {
+        int k;
+        const int j = src.point(base + lane, k);
+        const float sx = loc[j].x + (float)(k - 1) * d;
+        const MirrorVal v = mirror_value(mx - sx, my + yabs[j], kf, K, tau);
+        sv[warp][lane] = make_float4(v.ur, v.ui, v.gxr, v.gxi);
+        sw[warp][lane] = make_float2(v.gyr, v.gyi);
+        sj[warp][lane] = j;
       }
-      __syncthreads();
-      const int cnt = min(kMirSrc, ns - base);
-      mirror_batch(src, cnt, warp, kEvWarps, me.x, me.y, kap, K, tau, acc);
+      __syncwarp();
+      for (int e = 0; e < cnt; ++e) {
+        const float4 a = sv[warp][e];
+        const float2 b2 = sw[warp][e];
+        const MirrorVal v{a.x, a.y, a.z, a.w, b2.x, b2.y};
+        const float *q = qsm + (size_t)sj[warp][e] * rp;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          const int r = 32 * b + lane;
+          acc[b].add(r < nr ? __ldg(q + r) : 0.0f, v);
+        }
+      }
     }
-    red[warp][0][lane] = acc.li;
-    red[warp][1][lane] = acc.gix;
-    red[warp][2][lane] = acc.giy;
-    red[warp][3][lane] = acc.ur.x;
-    red[warp][4][lane] = acc.ur.y;
-    red[warp][5][lane] = acc.grx.x;
-    red[warp][6][lane] = acc.grx.y;
-    red[warp][7][lane] = acc.gry.x;
-    red[warp][8][lane] = acc.gry.y;
-    __syncthreads();
-    if (warp == 0 && act) {
-      float v[9];
-      for (int c = 0; c < 9; ++c) {
-        v[c] = 0.f;
-        for (int w = 0; w < kEvWarps; ++w) v[c] += red[w][c][lane];
-      }
-      const int64_t o = perm[i];
-      // assign: written before the leaf outputs, which then add it (split
-      // evaluation); otherwise added to the leaf outputs
-      const double w0 = (double)(v[0] * c4 + v[3] * i2pi), w1 = (double)(v[4] * i2pi);
-      pot[2 * o] = assign ? w0 : pot[2 * o] + w0;
-      pot[2 * o + 1] = assign ? w1 : pot[2 * o + 1] + w1;
-      if (grad) {
-        const double g0 = (double)((v[1] + v[5]) * i2pi), g1 = (double)(v[6] * i2pi);
-        const double g2 = (double)((v[2] + v[7]) * i2pi), g3 = (double)(v[8] * i2pi);
-        grad[4 * o + 0] = assign ? g0 : grad[4 * o + 0] + g0;
-        grad[4 * o + 1] = assign ? g1 : grad[4 * o + 1] + g1;
-        grad[4 * o + 2] = assign ? g2 : grad[4 * o + 2] + g2;
-        grad[4 * o + 3] = assign ? g3 : grad[4 * o + 3] + g3;
-      }
+    const int64_t o = perm[i];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const int r = 32 * b + lane;
+      if (r < nr)
+        acc[b].put(pot + (size_t)r * rs.out, grad ? grad + 2 * (size_t)r * rs.out : nullptr, o, false);
     }
-    __syncthreads();
   }
 }
 
@@ -1932,7 +2024,7 @@ k_mirror_targets(const int64_t *__restrict__ list, const double *__restrict__ xt
                  const int *__restrict__ leaf_start, int H,
                  double x0, double side, double qscale, KappaLog K, float tau,
                  double *__restrict__ pot, double *__restrict__ grad) {
-  __shared__ float red[kEvWarps][9];
+  __shared__ float red[kEvWarps][6];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = list[blockIdx.x];
   const int nx = 1 << H;
@@ -1942,45 +2034,27 @@ k_mirror_targets(const int64_t *__restrict__ list, const double *__restrict__ xt
   const int ix = (int)(quantise(__dsub_rn(x, x0), side, qscale) >> (30 - H));
   const double2 c = leaf_centre_at(x0, dd, ix, 0);
   const float mx = (float)(x - c.x), my = (float)y;
-  const cf kap = mk((float)K.kappa.x, (float)K.kappa.y);
-  NearAcc acc;
-  acc.lf = acc.gx = acc.gy = acc.li = acc.gix = acc.giy = 0.f;
-  acc.ur = acc.grx = acc.gry = mk(0.f, 0.f);
+  const KappaF kf = kappa_f(K);
+  MirrorAcc acc;
+  acc.clear();
   for (int k = 0; k < 3; ++k) {
     const int sx = ix - 1 + k;
     if (sx < 0 || sx >= nx) continue;
     const uint64_t sl = box_morton(sx, 0);
     const int s0 = leaf_start[sl], s1 = leaf_start[sl + 1];
     const float ox = (float)(k - 1) * d;
-    for (int j = s0 + (int)threadIdx.x; j < s1; j += blockDim.x) {
-      const float2 v = loc[j];
-      mirror_pair(make_float4(v.x + ox, yabs[j], qs[j], 0.f), mx, my, kap, K, tau, acc);
-    }
+    for (int j = s0 + (int)threadIdx.x; j < s1; j += blockDim.x)
+      acc.add(qs[j], mirror_value(mx - (loc[j].x + ox), my + yabs[j], kf, K, tau));
   }
-  float v[9] = {acc.li,    acc.gix,   acc.giy,   acc.ur.x, acc.ur.y,
-                acc.grx.x, acc.grx.y, acc.gry.x, acc.gry.y};
-#pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    v[e] = warp_sum(v[e]);
-    if (lane == 0) red[warp][e] = v[e];
-  }
+  acc.reduce<32>(0xffffffffu);
+  if (lane == 0)
+    for (int e = 0; e < 6; ++e) red[warp][e] = acc.v[e];
   __syncthreads();
   if (threadIdx.x != 0) return;
-#pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    v[e] = 0.f;
-    for (int w = 0; w < kEvWarps; ++w) v[e] += red[w][e];
-  }
-  const float c4 = (float)(0.69314718055994530942 / (4.0 * HP_PI));
-  const float i2pi = (float)(1.0 / HP_TWO_PI);
-  pot[2 * t] += (double)(v[0] * c4 + v[3] * i2pi);
-  pot[2 * t + 1] += (double)(v[4] * i2pi);
-  if (grad) {
-    grad[4 * t + 0] += (double)((v[1] + v[5]) * i2pi);
-    grad[4 * t + 1] += (double)(v[6] * i2pi);
-    grad[4 * t + 2] += (double)((v[2] + v[7]) * i2pi);
-    grad[4 * t + 3] += (double)(v[8] * i2pi);
-  }
+  acc.clear();
+  for (int w = 0; w < kEvWarps; ++w)
+    for (int e = 0; e < 6; ++e) acc.v[e] += red[w][e];
+  acc.put(pot, grad, t, false);
 }
 
 inline unsigned cdiv_u(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
@@ -2034,10 +2108,9 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   // the plan's side stream runs the far-field passes; L2P joins them.  In
   // double precision the near field takes the single-precision pipe (near64.cu)
   // and the far field the FP64 pipe, so the two overlap.
-  const int nxl = 1 << H, tps = nxl >= kTl ? nxl / kTl : 1;
   const bool split = !mw && !tw;
   if (split && !((sizeof(R) == 4 ? (void *)pl->near : (void *)pl->near64) && pl->side_stream &&
-                 pl->ev_fork && pl->ev_join && pl->ev_gather)) {
+                 pl->m2l_stream && pl->ev_fork && pl->ev_join && pl->ev_gather && pl->ev_m2lh)) {
     set_last_error("plan without its near-field buffer or side stream");
     return HPFMM_ECUDA;
   }
@@ -2049,7 +2122,10 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   // image/reaction pairs and the mirror M2L (into separate arrays that the
   // downward pass adds) on the plan's high-priority m2l stream, joined into
   // the far-field chain (ev_m2lh) before the downward pass
-  const bool leaf_m2l_apart = split && H >= 3 && pl->m2l_stream && pl->ev_s2m && pl->ev_m2lh;
+  // (double precision: the far field stays in one chain, bound by the FP64 pipe
+  // as a whole, and the near field takes the m2l stream)
+  const bool leaf_m2l_apart =
+      sizeof(R) == 4 && split && H >= 3 && pl->m2l_stream && pl->ev_s2m && pl->ev_m2lh;
   const bool mirror_apart = leaf_m2l_apart && pl->mir_A && pl->ev_up;
   if (split) {
     HP_CUDA(cudaEventRecord(pl->ev_fork, st));
@@ -2060,24 +2136,37 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   // near field reads them through perm itself)
   pass_begin(pl, fs, PASS_GATHER);
   if (split)
-    k_gather_q<R><<<dim3(cdiv_u(n, 256), nr), 256, 0, fs>>>(q, pl->perm, n, qs, (R *)nullptr, 0,
-                                                           pl->qexp);
+    k_gather_q<R><<<dim3(cdiv_u(n, 256)), 256, 0, fs>>>(q, pl->perm, n, qs, pl->qexp);
+  else if (mw)
+    HP_CUDA(launch_dependent(k_gather_multi, dim3(cdiv_u(n, 32), cdiv_u(mw->rp, kGmR)),
+                             dim3(32 * kGmWarps), 0, st, q, pl->perm, n, nr, (float *)qs,
+                             (float *)mw->qsm, mw->rp));
   else
-    HP_CUDA(launch_dependent(k_gather_q<R>, dim3(cdiv_u(n, 256), nr), dim3(256), 0, st, q,
-                             pl->perm, n, qs, mw ? (R *)mw->qsm : (R *)nullptr, mw ? mw->rp : 0,
-                             (int *)nullptr));
+    HP_CUDA(launch_dependent(k_gather_q<R>, dim3(cdiv_u(n, 256)), dim3(256), 0, st, q, pl->perm, n,
+                             qs, (int *)nullptr));
   pass_end(pl, fs, PASS_GATHER, 1);
   if (split) {
     HP_CUDA(cudaEventRecord(pl->ev_gather, fs));
-    if (sizeof(R) == 8) HP_CUDA(cudaStreamWaitEvent(st, pl->ev_gather, 0));
-    pass_begin(pl, st, PASS_EVAL);
-    if (sizeof(R) == 8)
-      HP_TRY(near64_launch(pl, (const double *)qs, st));
-    else
-      HP_CUDA(launch_dependent(k_near32, dim3((unsigned)(tps * tps)), dim3(32 * kEvWarps), kTpSmem,
-                               st, pl->loc32, pl->loclo, q, pl->perm,
+    if (sizeof(R) == 8) {
+      // on a stream of the far field's priority (at the caller's it waited for
+      // the last of the far field's blocks: 2.6 ms instead of 1.1), its blocks
+      // limited to a part of each SM (near64_launch)
+      cudaStream_t ns = pl->m2l_stream;
+      HP_CUDA(cudaStreamWaitEvent(ns, pl->ev_gather, 0));
+      pass_begin(pl, ns, PASS_EVAL);
+      HP_TRY(near64_launch(pl, (const double *)qs, ns));
+      pass_end(pl, ns, PASS_EVAL, near64_kernels(pl));
+      HP_CUDA(cudaEventRecord(pl->ev_m2lh, ns));
+    } else {
+      // 2 x 2 tiles from 24 points a leaf (k_near32)
+      const int tl = (double)n >= 24.0 * (double)pl->nleaf ? 2 : kTl;
+      const int tps = (1 << H) >= tl ? (1 << H) / tl : 1;
+      pass_begin(pl, st, PASS_EVAL);
+      HP_CUDA(launch_dependent(tl == 2 ? k_near32<2> : k_near32<kTl>, dim3((unsigned)(tps * tps)),
+                               dim3(32 * kEvWarps), kTpSmem, st, pl->loc32, pl->loclo, q, pl->perm,
                                pl->leaf_start, H, dg, pl->near));
-    pass_end(pl, st, PASS_EVAL, sizeof(R) == 8 ? near64_kernels(pl) : 1);
+      pass_end(pl, st, PASS_EVAL, 1);
+    }
     // the bottom-row image/reaction sums need only the sources too: written
     // now, added by the L2P kernel.  On the m2l stream (idle until the S2M is
     // done), off the near field's stream, after the gather.
@@ -2087,10 +2176,10 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
     if (sizeof(R) == 8)
       HP_TRY(mirror64_launch(pl, (const double *)qs, pot, grad, ms));
     else
-      k_mirror32<<<dim3((unsigned)(1 << H), 1, kMirSplit), 32 * kEvWarps, 0, ms>>>(
+      k_mirror32<<<dim3((unsigned)(1 << H), 1, kMirSplit), kMirThreads, 0, ms>>>(
           pl->loc32, pl->yabs, (const float *)qs, pl->perm, pl->leaf_start, H, dg,
           kappa_log(pl->kre, pl->kim), pl->prec == HPFMM_MIXED ? (float)pl->tau_fp64 : 0.f, pot,
-          grad, rs, 1);
+          grad);
     pass_end(pl, ms, PASS_NEAR_MIRROR, 1);
   }
   pass_begin(pl, fs, PASS_P2M);
@@ -2104,18 +2193,22 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
     --ksub;
   const int l0 = H - ksub;
   if (sizeof(R) == 8) {
-    LeafPoints<double> lp{pl->xs, pl->ys, 0.0};
-    size_t shp2m = sizeof(cd) * P1 * 33 * kWarpsPerBlock;
-    k_p2m<double><<<cdiv_u(pl->nleaf, kWarpsPerBlock), 32 * kWarpsPerBlock, shp2m, fs>>>(
-        lp, (const double *)qs, pl->leaf_start, H, dg, p, (cd *)M);
+    const int nlb = pl->nleaf >= 16 * 256 ? 16 : (pl->nleaf >= 4 * 256 ? 4 : 1);
+    k_p2m64<<<cdiv_u(pl->nleaf, nlb), kP2mThreads, p2m64_smem(p), fs>>>(
+        pl->xs, pl->ys, (const double *)qs, pl->leaf_start, H, nlb, dg, p, (cd *)M);
   } else {
     if (mw)
       k_s2m_multi<kRhsChunk><<<dim3(cdiv_u((int64_t)pl->nleaf * P1, 256), mw->rp / kRhsChunk),
                                256, 0, fs>>>(pl->loc32, (const float *)mw->qsm, mw->rp, nr,
                                              pl->leaf_start, H, dg, p, (cf *)M, rs);
-    else
-      k_s2m_tile<<<cdiv_u(pl->nleaf, kS2mLeaves), kS2mThreads, 0, fs>>>(
-          pl->loc32, (const float *)qs, pl->leaf_start, H, dg, p, (cf *)M, rs);
+    else {
+      const int nlb = pl->nleaf >= 64 * 512 ? 64 : (pl->nleaf >= 16 * 256 ? 16 : 4);
+      const int items = nlb * ((P1 + kS2mGroup - 1) / kS2mGroup);
+      int S = 1;
+      while (S < 16 && 2 * S * items <= kS2mThreads) S *= 2;
+      k_s2m_tile<<<cdiv_u(pl->nleaf, nlb), kS2mThreads, 0, fs>>>(
+          pl->loc32, (const float *)qs, pl->leaf_start, H, nlb, S, dg, p, (cf *)M, rs);
+    }
   }
   pass_end(pl, fs, PASS_P2M, 1);
   // split single precision: the M2L of the leaf level needs only the leaf
@@ -2127,31 +2220,34 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
     HP_CUDA(cudaEventRecord(pl->ev_s2m, fs));
     HP_CUDA(cudaStreamWaitEvent(pl->m2l_stream, pl->ev_s2m, 0));
     pass_begin(pl, pl->m2l_stream, PASS_M2L_FREE);
-    leaf_m2l_done = launch_m2l_patch<R>(p, H, H, H, dg, (const cpx<R> *)pl->t_m2l_pad, logs, M,
-                                        A, B, pl->status, pl->m2l_stream, 1, rs, pl->leaf_start,
-                                        1);
+    leaf_m2l_done = launch_m2l_patch(p, H, H, H, dg, (const cpx<R> *)pl->t_m2l_pad, logs, M, A, B,
+                                     pl->status, pl->m2l_stream, 1, rs, pl->leaf_start, 1);
     pass_end(pl, pl->m2l_stream, PASS_M2L_FREE, leaf_m2l_done ? 1 : 0);
     if (!mirror_apart) HP_CUDA(cudaEventRecord(pl->ev_m2lh, pl->m2l_stream));
   }
   pass_begin(pl, fs, PASS_M2M);
-  // the subtree blocks; when every level above them is small, the last of
-  // them also runs those (levels l0 - 1 .. 1), otherwise the levels of 1024
-  // boxes and more get one launch each and the small top levels one block
-  const bool coarse_in_upward = ksub > 0 && l0 <= ksub;
+  // the subtree blocks; with few boxes above them the last of them also runs
+  // the levels l0 - 1 .. 1
+  const size_t sm_sub = ksub > 0 ? upward_smem<R>(p, ksub) : 0;
+  const bool all256 = (ksub >= 4 || (H <= 6 && nr == 1)) && upward_smem<R>(p, 4) <= kFusedSmem;
+  const size_t sm_top = upward_smem<R>(p, l0 < 3 ? l0 : (all256 && l0 == 4 ? 4 : 3));
+  const bool coarse_in_upward = ksub > 0 && l0 <= kCoarse;
   if (ksub > 0) {
-    size_t sm = upward_smem<R>(p, ksub);
+    const size_t sm = coarse_in_upward && sm_top > sm_sub ? sm_top : sm_sub;
     unsigned nb = (unsigned)(int64_t(1) << (2 * l0));
-    HP_CUDA(launch_dependent(k_upward<R>, dim3(nb, nr), dim3(256), sm, fs, H, ksub, p, Tm2m, M, rs,
+    HP_CUDA(launch_dependent(k_upward<R>, dim3(nb, nr), dim3(256), sm, fs, H, ksub,
+                             all256 ? 256 : 64, p, Tm2m, M, rs,
                              coarse_in_upward ? pl->ctr : (int *)nullptr));
   }
   int nm2m = ksub > 0 ? 1 : 0;
   if (!coarse_in_upward) {
-    for (int l = l0 - 1; l >= kCoarseBig; --l, ++nm2m)
+    const int top = l0 < kCoarse ? l0 : kCoarse;  // the level the one block starts from
+    for (int l = l0 - 1; l >= top; --l, ++nm2m)
       k_m2m_level<R><<<dim3(cdiv_u((int64_t(1) << (2 * l)) * P1, 256), nr), 256, 0, fs>>>(
           l, p, Tm2m, M, rs);
-    const int lsmall = l0 - 1 < kCoarseBig - 1 ? l0 - 1 : kCoarseBig - 1;
-    if (lsmall >= 1) {
-      k_m2m_coarse<R><<<dim3(1, nr), 1024, 0, fs>>>(lsmall, p, Tm2m, M, rs);
+    if (top > 1) {
+      k_m2m_coarse<R><<<dim3(1, nr), 512, upward_smem<R>(p, top < 3 ? top : 3), fs>>>(top, p, Tm2m,
+                                                                                      M, rs);
       ++nm2m;
     }
   }
@@ -2182,9 +2278,9 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
       tc_m2l = patched = launch_m2l_tc(p, H, dg, (const float *)pl->t_m2l_tc, logs, (const cf *)M, (cf *)A,
                               (cf *)B, pl->status, fs, nr, rs);
     if (!patched)
-      patched = launch_m2l_patch<R>(p, H, 2, leaf_m2l_done ? H - 1 : H, dg,
-                                    (const cpx<R> *)pl->t_m2l_pad, logs, M, A, B, pl->status, fs,
-                                    nr, rs, pl->leaf_start, tw ? 0 : 1);
+      patched = launch_m2l_patch(p, H, 2, leaf_m2l_done ? H - 1 : H, dg,
+                                 (const cpx<R> *)pl->t_m2l_pad, logs, M, A, B, pl->status, fs, nr,
+                                 rs, pl->leaf_start, tw ? 0 : 1);
     pass_end(pl, fs, PASS_M2L_FREE, patched ? (tc_m2l ? H - 1 : 1) : 0);
   }
   // the leaf level's M2L joins the chain here (the mirror M2L below adds to
@@ -2226,8 +2322,11 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   if (split) {
     HP_CUDA(cudaEventRecord(pl->ev_join, fs));
     HP_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
-    int kd = H - 1 < 3 ? H - 1 : 3;  // subtrees of 64 leaves: 4^(H-3) blocks
-    while (kd > 0 && downward_smem<R>(p, kd, true) > kFusedSmem) --kd;
+    if (sizeof(R) == 8) HP_CUDA(cudaStreamWaitEvent(st, pl->ev_m2lh, 0));
+    // subtrees of 64 leaves, smaller ones where that leaves fewer blocks than
+    // SMs (40009 points at p = 24, level 5: 520 us with 16 blocks)
+    int kd = H - 1 < 3 ? H - 1 : 3;
+    while (kd > 0 && (downward_smem<R>(p, kd, true) > kFusedSmem || 2 * (H - kd) < 8)) --kd;
     pass_begin(pl, st, PASS_L2L);
     const DownEval ev{pl->loc32, pl->near, pl->xs,  pl->ys, pl->near64, n, pl->qexp,
                       pl->perm,  pl->keys, dg, pot, grad};
@@ -2278,9 +2377,10 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
                                  grad);
     pass_end(pl, st, PASS_EVAL, 1);
     pass_begin(pl, st, PASS_NEAR_MIRROR);
-    k_mirror32<<<dim3((unsigned)(1 << H), nr, kMirSplit), 32 * kEvWarps, 0, st>>>(
-        pl->loc32, pl->yabs, (const float *)qs, pl->perm, pl->leaf_start, H, dg,
-        kappa_log(pl->kre, pl->kim), tau, pot, grad, rs, 0);
+    auto *mir = nr > 32 ? k_mirror32m<64> : k_mirror32m<32>;
+    mir<<<dim3((unsigned)(1 << H), 1, kMirSplit), 32 * kMirmWarps, 0, st>>>(
+        pl->loc32, pl->yabs, (const float *)mw->qsm, mw->rp, nr, pl->perm, pl->leaf_start, H, dg,
+        kappa_log(pl->kre, pl->kim), tau, pot, grad, rs);
     pass_end(pl, st, PASS_NEAR_MIRROR, 1);
   }
   HP_LAUNCH_CHECK();
@@ -2290,19 +2390,42 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
 }  // namespace
 
 size_t fmm_shared_bytes_max(int p, bool fp64) {
-  size_t c = fp64 ? sizeof(cd) : sizeof(cf);
-  size_t P1 = p + 1;
-  size_t a = c * P1 * 33 * kWarpsPerBlock, b = c * (P1 * P1 + P1 * 33);
-  return a > b ? a : b;
+  const size_t P1 = p + 1;
+  return (fp64 ? sizeof(cd) : sizeof(cf)) * (P1 * P1 + P1 * 33);
 }
 
 hpfmm_status fmm_set_smem_limits(int p) {
   size_t s64 = fmm_shared_bytes_max(p, true), s32 = fmm_shared_bytes_max(p, false);
-  HP_CUDA(cudaFuncSetAttribute(k_p2m<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64));
-  HP_CUDA(cudaFuncSetAttribute(k_p2m<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32));
+  // (the kernels of the split evaluation; those of the one-stream forms keep
+  // the default split, with more L1)
+  HP_CUDA(prefer_shared(k_gather_q<float>));
+  HP_CUDA(prefer_shared(k_gather_q<double>));
+  HP_CUDA(prefer_shared(k_p2m64));
+  HP_CUDA(prefer_shared(k_s2m_tile));
+  HP_CUDA(prefer_shared(k_upward<float>));
+  HP_CUDA(prefer_shared(k_upward<double>));
+  HP_CUDA(prefer_shared(k_m2m_coarse<float>));
+  HP_CUDA(prefer_shared(k_m2m_coarse<double>));
+  HP_CUDA(prefer_shared(k_m2m_level<float>));
+  HP_CUDA(prefer_shared(k_m2m_level<double>));
+  HP_CUDA(prefer_shared(k_m2l_mirror_all<float>));
+  HP_CUDA(prefer_shared(k_m2l_mirror_all<double>));
+  HP_CUDA(prefer_shared(k_downward<float, true>));
+  HP_CUDA(prefer_shared(k_downward<double, true>));
+  HP_CUDA(prefer_shared(k_near32<2>));
+  HP_CUDA(prefer_shared(k_near32<kTl>));
+  HP_CUDA(prefer_shared(k_mirror32));
+  HP_CUDA(cudaFuncSetAttribute(k_p2m64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)p2m64_smem(p)));
   HP_CUDA(cudaFuncSetAttribute(k_m2l_free<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64));
-  HP_CUDA(cudaFuncSetAttribute(k_near32, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  HP_CUDA(cudaFuncSetAttribute(k_near32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kTpSmem));
+  HP_CUDA(cudaFuncSetAttribute(k_near32<kTl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kTpSmem));
+  HP_CUDA(cudaFuncSetAttribute(k_m2m_coarse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kFusedSmem));
+  HP_CUDA(cudaFuncSetAttribute(k_m2m_coarse<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kFusedSmem));
   HP_CUDA(cudaFuncSetAttribute(k_upward<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kFusedSmem));
   HP_CUDA(cudaFuncSetAttribute(k_upward<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -28,48 +28,152 @@ __device__ __forceinline__ double f2d(float v) {
   return __longlong_as_double((long long)r);
 }
 
+// single-precision sums of one target's free-space pairs
 struct NearAcc {
-  float lf, gx, gy;                 // free: sum q log2 r^2, sum q (dx, dy) / r^2
-  float li, gix, giy;               // image
-  cf ur, grx, gry;                  // reaction (pairs evaluated in single or double)
+  float lf, gx, gy;  // sum q log2 r^2, sum q (dx, dy) / r^2
 };
 
-// one image + reaction pair of a bottom-row target (x in its leaf frame, y
-// itself) and a bottom-row source s = (x in the same frame, y itself, q):
-// single precision where the series is accurate, else double.  The y values
-// are not taken from the leaf frames: near the boundary Y = y_i + y_j would
-// lose its relative precision to the rounding of the leaf offsets.
-__device__ __forceinline__ void mirror_pair(const float4 s, float mx, float my, cf kap,
-                                            const KappaLog &K, float tau, NearAcc &a) {
-  float dx = mx - s.x;
-  float Y = my + s.y;
-  float R2 = fmaf(dx, dx, Y * Y);
-  float qi = s.z * fast_rcp(R2);
-  a.li = fmaf(s.z, __log2f(R2), a.li);
-  a.gix = fmaf(qi, dx, a.gix);
-  a.giy = fmaf(qi, Y, a.giy);
-  cf sp_ = mk(Y, -dx), sm_ = mk(Y, dx);
-  cf Pp = kap * sp_, Pm = kap * sm_;
-  if (abs2(Pp) <= 1.f && Y >= tau) {
-    cf J0p, J1p, J0m, J1m;
-    j01_f(Pp, J0p, J1p);
-    j01_f(Pm, J0m, J1m);
-    a.ur = a.ur + s.z * (J0p + J0m);
-    cf tp = cdiv(J1p, sp_), tm = cdiv(J1m, sm_);
-    a.grx = a.grx + s.z * mul_i(tp - tm);
-    a.gry = a.gry - s.z * (tp + tm);
-  } else {
-    const double X = dx, Yd = Y;
-    cd J0p, J1p, J0m, J1m;
-    const double s2 = X * X + Yd * Yd;
-    j01_pm(K, X, Yd, s2, log(s2), J0p, J1p, J0m, J1m);
-    const double q = s.z;
-    // J_1 / s+- with s+- = Y -+ iX: one reciprocal of |s|^2 for both
-    const double inv = 1.0 / s2;
-    const cd tp = inv * (J1p * mk(Yd, X)), tm = inv * (J1m * mk(Yd, -X));
-    a.ur = a.ur + to<float>(q * (J0p + J0m));
-    a.grx = a.grx + to<float>(q * mul_i(tp - tm));
-    a.gry = a.gry - to<float>(q * (tp + tm));
-  }
+// The image and reaction pair of two points of the bottom leaf row for a unit
+// charge: u and its gradient, with the 1/2pi and 1/4pi factors.  They do not
+// depend on the charge, so many charge vectors share one evaluation.
+struct MirrorVal {
+  float ur, ui, gxr, gxi, gyr, gyi;
+};
+
+// in double precision, rounded: out of line, as the single-precision kernels
+// need it for few pairs
+static __device__ __noinline__ MirrorVal mirror_value_d(const KappaLog &K, double X, double Y) {
+  const double s2 = X * X + Y * Y, ln = log(s2), inv = 1.0 / s2;
+  cd J0p, J1p, J0m, J1m;
+  j01_pm(K, X, Y, s2, ln, J0p, J1p, J0m, J1m);
+  const double i2pi = 1.0 / HP_TWO_PI, w = i2pi * inv;
+  const cd tp = J1p * mk(Y, X), tm = J1m * mk(Y, -X);  // J_1 / s+- times s2
+  MirrorVal v;
+  v.ur = (float)(i2pi * (0.5 * ln + J0p.x + J0m.x));
+  v.ui = (float)(i2pi * (J0p.y + J0m.y));
+  v.gxr = (float)(w * (X - (tp.y - tm.y)));
+  v.gxi = (float)(w * (tp.x - tm.x));
+  v.gyr = (float)(w * (Y - (tp.x + tm.x)));
+  v.gyi = (float)(-w * (tp.y + tm.y));
+  return v;
 }
 
+// kappa as the single-precision pair uses it
+struct KappaF {
+  cf kappa;
+  float a2, lk, ak;  // |kappa|^2, ln |kappa|, arg kappa
+  bool real;
+};
+__device__ __forceinline__ KappaF kappa_f(const KappaLog &K) {
+  return KappaF{mk((float)K.kappa.x, (float)K.kappa.y), (float)abs2(K.kappa), (float)K.lk,
+                (float)K.ak, K.kappa.y == 0.0};
+}
+
+// e^{-P} and sum_{k=1}^{11} P^k/(k k!) in single precision, P2 = |P|^2 <= 1, by
+// the real recurrence of real_poly
+__device__ __forceinline__ void exp_sum_f(cf P, float P2, cf &E, cf &S) {
+  const float c[11] = {1.0f,           1.0f / 4.0f,      1.0f / 18.0f,     1.0f / 96.0f,
+                       1.0f / 600.0f,  1.0f / 4320.0f,   1.0f / 35280.0f,  1.0f / 322560.0f,
+                       1.0f / 3265920.0f, 1.0f / 36288000.0f, 1.0f / 439084800.0f};
+  float b1 = c[10], b2 = 0.0f;
+  const float r = P.x + P.x;
+#pragma unroll
+  for (int k = 9; k >= 1; --k) {
+    const float t = fmaf(r, b1, fmaf(-P2, b2, c[k]));
+    b2 = b1;
+    b1 = t;
+  }
+  S = P * mk(fmaf(P.x, b1, fmaf(-P2, b2, c[0])), P.y * b1);
+  const float e = __expf(-P.x);
+  float sn, cs;
+  __sincosf(-P.y, &sn, &cs);
+  E = mk(e * cs, e * sn);
+}
+
+// Single precision where the series is accurate (|P| <= 1) and the pair is not
+// below tau, else double.  X the difference of the x, Y the sum of the y.  ln
+// and reciprocal of X^2 + Y^2 serve the image and both reaction terms, and for
+// real kappa the arguments P+- are conjugate, J_n(conj P) = conj J_n(P) + 2 pi i
+// conj(P)^n e^{-conj P}: about 130 instructions a pair (two complex series, four
+// divisions and the accumulation for one charge took about 450).
+__device__ __forceinline__ MirrorVal mirror_value(float X, float Y, const KappaF &kf,
+                                                  const KappaLog &K, float tau) {
+  const float s2 = fmaf(X, X, Y * Y), P2 = kf.a2 * s2;
+  if (!(P2 <= 1.0f && Y >= tau))
+    return mirror_value_d(K, X, Y);
+  const float ln = 0.693147180559945f * fast_lg2(s2), inv = fast_rcp(s2);
+  const float lr = fmaf(0.5f, ln, kf.lk), th = atan2f(X, Y);
+  const float g = -(float)HP_EULER_GAMMA - lr, pi = (float)HP_PI;
+  const cf Pp = kf.kappa * mk(Y, -X), Pm = kf.kappa * mk(Y, X);
+  cf Ep, Sp, Em, Sm;
+  exp_sum_f(Pp, P2, Ep, Sp);
+  if (kf.real) {
+    Em = conj(Ep);
+    Sm = conj(Sp);
+  } else {
+    exp_sum_f(Pm, P2, Em, Sm);
+  }
+  const cf J0p = Ep * mk(g - Sp.x, pi - (kf.ak - th) - Sp.y);
+  const cf J0m = Em * mk(g - Sm.x, pi - (kf.ak + th) - Sm.y);
+  cf J1p = Pp * J0p, J1m = Pm * J0m;
+  J1p.x += 1.0f;
+  J1m.x += 1.0f;
+  const cf tp = J1p * mk(Y, X), tm = J1m * mk(Y, -X);
+  const float i2pi = (float)(1.0 / HP_TWO_PI), w = i2pi * inv;
+  MirrorVal v;
+  v.ur = i2pi * (0.5f * ln + (J0p.x + J0m.x));
+  v.ui = i2pi * (J0p.y + J0m.y);
+  v.gxr = w * (X - (tp.y - tm.y));
+  v.gxi = w * (tp.x - tm.x);
+  v.gyr = w * (Y - (tp.x + tm.x));
+  v.gyi = -w * (tp.y + tm.y);
+  return v;
+}
+
+// sums over the sources of one target
+struct MirrorAcc {
+  float v[6];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int e = 0; e < 6; ++e) v[e] = 0.0f;
+  }
+  __device__ __forceinline__ void add(float q, const MirrorVal &m) {
+    v[0] = fmaf(q, m.ur, v[0]);
+    v[1] = fmaf(q, m.ui, v[1]);
+    v[2] = fmaf(q, m.gxr, v[2]);
+    v[3] = fmaf(q, m.gxi, v[3]);
+    v[4] = fmaf(q, m.gyr, v[4]);
+    v[5] = fmaf(q, m.gyi, v[5]);
+  }
+  // over the G lanes of an aligned group
+  template <int G>
+  __device__ __forceinline__ void reduce(unsigned mask) {
+#pragma unroll
+    for (int e = 0; e < 6; ++e)
+#pragma unroll
+      for (int o = G / 2; o > 0; o >>= 1) v[e] += __shfl_xor_sync(mask, v[e], o);
+  }
+  // to the outputs of point o: assigned, or added to what is there
+  __device__ __forceinline__ void put(double *pot, double *grad, int64_t o, bool assign) const {
+    double2 *po = reinterpret_cast<double2 *>(pot) + o;
+    double2 *go = reinterpret_cast<double2 *>(grad) + 2 * o;
+    double2 a = make_double2(f2d(v[0]), f2d(v[1]));
+    double2 b = make_double2(f2d(v[2]), f2d(v[3])), c = make_double2(f2d(v[4]), f2d(v[5]));
+    if (!assign) {
+      const double2 t = *po;
+      a.x += t.x;
+      a.y += t.y;
+    }
+    *po = a;
+    if (!grad) return;
+    if (!assign) {
+      const double2 t = go[0], u = go[1];
+      b.x += t.x;
+      b.y += t.y;
+      c.x += u.x;
+      c.y += u.y;
+    }
+    go[0] = b;
+    go[1] = c;
+  }
+};

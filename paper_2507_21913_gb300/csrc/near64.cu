@@ -111,73 +111,74 @@ k_near64(const double *__restrict__ xs, const double *__restrict__ ys,
     for (int e = threadIdx.x; e < kFfLogN; e += blockDim.x) tab[e] = g_log_tab[e];
     __syncthreads();
   }
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int g = (int)(threadIdx.x & (S - 1));
-  const int64_t ti = t / S;
-  const bool act = ti < n;
-  const int i = act ? (int)ti : 0;
-  double lf = 0.0, gx = 0.0, gy = 0.0;
-  if (act) {
-    const uint64_t leaf = keys[i] >> (60 - 2 * H);
-    NearWalk w;
-    w.start(leaf_start, box_ix(leaf), box_iy(leaf), 1 << H, g);
-    if (fast) {
-      // r^2 in units of 2^(2 kd - 46): the exponent's part of the log
-      const int ebias = 46 - 2 * leaf_exponent(dg, H);
-      const longlong2 me = fxy[i];
-      ff_sum3 sl{0.f, 0.f, 0.f}, sk{0.f, 0.f, 0.f}, sx{0.f, 0.f, 0.f}, sy{0.f, 0.f, 0.f};
-      for (; w.more(); w.step(S)) {
-        const longlong2 s = fxy[w.k];
-        const float2 qv = fq[w.k];
-        const int64_t DX = me.x - s.x, DY = me.y - s.y;
-        const int hx = (int)(DX >> 32), hy = (int)(DY >> 32);
-        if (((hx ^ (hx >> 31)) | (hy ^ (hy >> 31))) == 0) {
-          // closer than 2^-28 of the leaf side, where the fixed-point unit
-          // could show, or the target itself
-          if (w.k != i) {
-            const double dx = xs[i] - xs[w.k], dy = ys[i] - ys[w.k];
-            PairAcc<double> a;
-            pair_free(a, dx, dy, qs[w.k]);
-            lf += a.lf;
-            gx += a.gfx;
-            gy += a.gfy;
+  const int g = (int)(threadIdx.x & (S - 1)), per = (int)blockDim.x / S;
+  for (int64_t t0 = (int64_t)blockIdx.x * per; t0 < n; t0 += (int64_t)gridDim.x * per) {
+    const int64_t ti = t0 + (int)threadIdx.x / S;
+    const bool act = ti < n;
+    const int i = act ? (int)ti : 0;
+    double lf = 0.0, gx = 0.0, gy = 0.0;
+    if (act) {
+      const uint64_t leaf = keys[i] >> (60 - 2 * H);
+      NearWalk w;
+      w.start(leaf_start, box_ix(leaf), box_iy(leaf), 1 << H, g);
+      if (fast) {
+        // r^2 in units of 2^(2 kd - 46): the exponent's part of the log
+        const int ebias = 46 - 2 * leaf_exponent(dg, H);
+        const longlong2 me = fxy[i];
+        ff_sum3 sl{0.f, 0.f, 0.f}, sk{0.f, 0.f, 0.f}, sx{0.f, 0.f, 0.f}, sy{0.f, 0.f, 0.f};
+        for (; w.more(); w.step(S)) {
+          const longlong2 s = fxy[w.k];
+          const float2 qv = fq[w.k];
+          const int64_t DX = me.x - s.x, DY = me.y - s.y;
+          const int hx = (int)(DX >> 32), hy = (int)(DY >> 32);
+          if (((hx ^ (hx >> 31)) | (hy ^ (hy >> 31))) == 0) {
+            // closer than 2^-28 of the leaf side, where the fixed-point unit
+            // could show, or the target itself
+            if (w.k != i) {
+              const double dx = xs[i] - xs[w.k], dy = ys[i] - ys[w.k];
+              PairAcc<double> a;
+              pair_free(a, dx, dy, qs[w.k]);
+              lf += a.lf;
+              gx += a.gfx;
+              gy += a.gfy;
+            }
+            continue;
           }
-          continue;
+          const ff dx = ff_from_fixed(DX), dy = ff_from_fixed(DY), q{qv.x, qv.y};
+          const ff r2 = ff_norm2(dx, dy);
+          const float c = ff_rcp_approx(r2.h);
+          float k;
+          sl.add(ff_prod(ff_log(r2, c, tab, ebias, k), q));
+          sk.add(ff_prod(ff{k, 0.f}, q));
+          const ff qw = ff_prod(ff_recip(r2, c), q);
+          sx.add(ff_prod(qw, dx));
+          sy.add(ff_prod(qw, dy));
         }
-        const ff dx = ff_from_fixed(DX), dy = ff_from_fixed(DY), q{qv.x, qv.y};
-        const ff r2 = ff_norm2(dx, dy);
-        const float c = ff_rcp_approx(r2.h);
-        float k;
-        sl.add(ff_prod(ff_log(r2, c, tab, ebias, k), q));
-        sk.add(ff_prod(ff{k, 0.f}, q));
-        const ff qw = ff_prod(ff_recip(r2, c), q);
-        sx.add(ff_prod(qw, dx));
-        sy.add(ff_prod(qw, dy));
+        const double us = ldexp(1.0, qe - 1023);
+        const double ug = ldexp(1.0, qe - 1023 + 23 - leaf_exponent(dg, H));
+        lf += us * fma(0.69314718055994530942, sk.value(), sl.value());
+        gx += ug * sx.value();
+        gy += ug * sy.value();
+      } else {
+        PairAcc<double> a;
+        const double x = xs[i], y = ys[i];
+        for (; w.more(); w.step(S))
+          if (w.k != i) pair_free(a, x - xs[w.k], y - ys[w.k], qs[w.k]);
+        lf = a.lf;
+        gx = a.gfx;
+        gy = a.gfy;
       }
-      const double us = ldexp(1.0, qe - 1023);
-      const double ug = ldexp(1.0, qe - 1023 + 23 - leaf_exponent(dg, H));
-      lf += us * fma(0.69314718055994530942, sk.value(), sl.value());
-      gx += ug * sx.value();
-      gy += ug * sy.value();
-    } else {
-      PairAcc<double> a;
-      const double x = xs[i], y = ys[i];
-      for (; w.more(); w.step(S))
-        if (w.k != i) pair_free(a, x - xs[w.k], y - ys[w.k], qs[w.k]);
-      lf = a.lf;
-      gx = a.gfx;
-      gy = a.gfy;
     }
-  }
-  for (int o = S >> 1; o > 0; o >>= 1) {
-    lf += __shfl_xor_sync(0xffffffffu, lf, o);
-    gx += __shfl_xor_sync(0xffffffffu, gx, o);
-    gy += __shfl_xor_sync(0xffffffffu, gy, o);
-  }
-  if (act && g == 0) {
-    near[i] = lf;
-    near[n + i] = gx;
-    near[2 * n + i] = gy;
+    for (int o = S >> 1; o > 0; o >>= 1) {
+      lf += __shfl_xor_sync(0xffffffffu, lf, o);
+      gx += __shfl_xor_sync(0xffffffffu, gx, o);
+      gy += __shfl_xor_sync(0xffffffffu, gy, o);
+    }
+    if (act && g == 0) {
+      near[i] = lf;
+      near[n + i] = gx;
+      near[2 * n + i] = gy;
+    }
   }
 }
 
@@ -263,6 +264,10 @@ hpfmm_status near64_prepare() {
   static ff tab[kFfLogN];
   ff_log_table(tab);
   HP_CUDA(cudaMemcpyToSymbol(g_log_tab, tab, sizeof tab));
+  HP_CUDA(prefer_shared(k_prep64));
+  HP_CUDA(prefer_shared(k_near64<true>));
+  HP_CUDA(prefer_shared(k_near64<false>));
+  HP_CUDA(prefer_shared(k_mirror64));
   done[dev] = true;
   return special_init_here();
 }
@@ -275,6 +280,10 @@ namespace {
 // field, take FP64 pairs.
 bool near64_fast(const hpfmm_plan *pl) { return pl->p <= 28 && pl->H >= 2; }
 }  // namespace
+
+// Blocks per SM of the float-pair kernel, which loops over the targets: the far
+// field's kernels, bound by the FP64 pipe with few warps, find room beside them.
+constexpr int kNearBlocks = 5;
 
 int near64_kernels(const hpfmm_plan *pl) { return near64_fast(pl) ? 2 : 1; }
 
@@ -289,7 +298,8 @@ hpfmm_status near64_launch(hpfmm_plan *pl, const double *qs, cudaStream_t st) {
     k_prep64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pl->xs, pl->ys, qs, n, pl->H, pl->dgeom,
                                                           pl->qexp, (longlong2 *)pl->fxy,
                                                           (float2 *)pl->fq);
-    k_near64<true><<<nb, 128, 0, st>>>(pl->xs, pl->ys, qs, (const longlong2 *)pl->fxy,
+    const unsigned most = (unsigned)(kNearBlocks * pl->sms);
+    k_near64<true><<<nb < most ? nb : most, 128, 0, st>>>(pl->xs, pl->ys, qs, (const longlong2 *)pl->fxy,
                                        (const float2 *)pl->fq, pl->keys, pl->leaf_start, n, pl->H,
                                        S, pl->dgeom, pl->qexp, pl->near64);
   } else {

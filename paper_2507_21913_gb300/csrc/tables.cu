@@ -83,7 +83,7 @@ __global__ void k_m2m_l2l(int p, cd *m2m, cd *l2l) {
 }
 
 // log-kernel M2L matrix for displacement t (scaled): T[l][k]
-__device__ void log_m2l_fill(cd t, int p, cd *T) {
+__device__ void log_m2l_fill(cd t, int p, cd *T, bool lcol) {
   int P1 = p + 1;
   cd ti = cinv(t);
   for (int e = threadIdx.x; e < P1 * P1; e += blockDim.x) {
@@ -97,7 +97,7 @@ __device__ void log_m2l_fill(cd t, int p, cd *T) {
       for (int j = 0; j < k + l; ++j) tp = tp * ti;
       v = c * tp;
     }
-    T[e] = v;
+    T[lcol ? k * P1 + l : e] = v;  // lcol: the output order l last
   }
 }
 
@@ -107,7 +107,7 @@ __global__ void k_free_m2l(int p, cd *T, cd *logt) {
   int P1 = p + 1;
   cd t = mk(-(double)dx, -(double)dy);
   if (dx == 0 && dy == 0) t = mk(1.0, 0.0);  // unused class
-  log_m2l_fill(t, p, T + (size_t)cls * P1 * P1);
+  log_m2l_fill(t, p, T + (size_t)cls * P1 * P1, false);
   if (threadIdx.x == 0) logt[cls] = clog_d(t);
 }
 
@@ -116,11 +116,12 @@ __global__ void k_img_m2l(int p, cd *T, cd *logt) {
   int dx = cls % 7 - 3, ysum = cls / 7 + 1;
   int P1 = p + 1;
   cd t = mk(-(double)dx, (double)ysum);
-  log_m2l_fill(t, p, T + (size_t)cls * P1 * P1);
+  log_m2l_fill(t, p, T + (size_t)cls * P1 * P1, true);
   if (threadIdx.x == 0) logt[cls] = clog_d(t);
 }
 
-// reaction M2L matrices Tr[level][cls][sign][n][m].  The Phi_2^- matrix of
+// reaction M2L matrices Tr[level][cls][sign][m][n] (output order n last: the
+// lanes of the mirror M2L take one n each).  The Phi_2^- matrix of
 // offset dx uses I_k at (+dx d, Y), which is the argument of the Phi_2^+
 // matrix of offset -dx; so a block owns one (level, ysum, m) with
 // shat = ysum + i m, evaluates It_k = J_k(P) / (2 pi k! shat^k) (thread k,
@@ -152,7 +153,7 @@ __global__ void k_reaction_m2l(int p, int H, const double *__restrict__ geo, cd 
   cd *outp = Tr + ((size_t)((lev - 1) * 21 + cls_p) * 2 + 0) * P1 * P1;
   cd *outm = Tr + ((size_t)((lev - 1) * 21 + cls_m) * 2 + 1) * P1 * P1;
   for (int e = threadIdx.x; e < P1 * P1; e += blockDim.x) {
-    const int n = e / P1, m = e % P1;
+    const int m = e / P1, n = e % P1;
     const cd v = Cb[(n + m) * (2 * p + 2) + m] * h[n + m];
     cd vp = v, vm = v;
     for (int r = 0; r < ((n - m) & 3); ++r) vp = mul_i(vp);  // i^{n-m}
@@ -274,6 +275,11 @@ hpfmm_status tables_static(hpfmm_plan *pl, cudaStream_t st) {
     k_m2l_pad<double><<<40, 64, 0, st>>>(p, (cd *)pl->t_m2l_pad);
     HP_LAUNCH_CHECK();
   }
+  return HPFMM_OK;
+}
+
+hpfmm_status tables_prepare() {
+  HP_CUDA(prefer_shared(k_reaction_m2l));
   return HPFMM_OK;
 }
 
