@@ -949,7 +949,10 @@ hpfmm_status adaptive_build(hpfmm_plan *pl, const double *x, const double *y, cu
   return HPFMM_OK;
 }
 
-hpfmm_status adaptive_prepare() { return special_init_here(); }
+hpfmm_status adaptive_prepare() {
+  HP_TRY(mirror_tables_here());
+  return special_init_here();
+}
 
 hpfmm_status adaptive_eval(hpfmm_plan *pl, const double *q, double *pot, double *grad,
                            cudaStream_t st) {

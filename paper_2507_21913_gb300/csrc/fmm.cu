@@ -2442,7 +2442,10 @@ hpfmm_status fmm_set_smem_limits(int p) {
   return HPFMM_OK;
 }
 
-hpfmm_status fmm_prepare() { return special_init_here(); }
+hpfmm_status fmm_prepare() {
+  HP_TRY(mirror_tables_here());
+  return special_init_here();
+}
 
 hpfmm_status fmm_eval(hpfmm_plan *pl, const double *q, double *pot, double *grad,
                       cudaStream_t st) {

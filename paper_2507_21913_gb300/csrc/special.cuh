@@ -29,6 +29,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "mirror_ff.cuh"
 
 #define HP_EULER_GAMMA 0.57721566490153286061
 #define HP_PI 3.14159265358979323846
@@ -174,12 +175,14 @@ __device__ inline cd jn_direct_single(cd P, int n) {
 struct KappaLog {
   cd kappa;
   double lk, ak;
+  KappaFF f;  // the same in float pairs
 };
 inline KappaLog kappa_log(double kre, double kim) {
   KappaLog K;
   K.kappa = mk(kre, kim);
   K.lk = 0.5 * log(kre * kre + kim * kim);
   K.ak = atan2(kim, kre);
+  K.f = KappaFF{ff_of(kre), ff_of(kim), ff_of(K.lk), ff_of(K.ak), kim == 0.0};
   return K;
 }
 
