@@ -2415,8 +2415,9 @@ hpfmm_status fmm_set_smem_limits(int p) {
   HP_CUDA(prefer_shared(k_near32<2>));
   HP_CUDA(prefer_shared(k_near32<kTl>));
   HP_CUDA(prefer_shared(k_mirror32));
+  // (the highest order's: plans of several orders live beside one another)
   HP_CUDA(cudaFuncSetAttribute(k_p2m64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)p2m64_smem(p)));
+                               (int)p2m64_smem(HPFMM_MAX_P)));
   HP_CUDA(cudaFuncSetAttribute(k_m2l_free<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64));
   HP_CUDA(cudaFuncSetAttribute(k_near32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kTpSmem));

@@ -91,3 +91,16 @@ def test_a_plan_forgets_earlier_charges():
     hp.hpfmm_eval(plan, t(1e200 * q))
     u2, g2 = hp.hpfmm_eval(plan, t(q))
     assert torch.equal(u, u2) and torch.equal(g, g2)
+
+
+@pytest.mark.parametrize("first,second", [(40, 4), (24, 12)])
+def test_plans_of_several_orders(first, second):
+    """A later plan of a lower order must not take shared memory from an
+    earlier plan's kernels."""
+    x, y, q = workloads.uniform(3001, seed=7)
+    a = hp.hpfmm_create(t(x), t(y), p=first, leaf_size=32)
+    u, g = hp.hpfmm_eval(a, t(q))
+    b = hp.hpfmm_create(t(x), t(y), p=second, leaf_size=32)
+    hp.hpfmm_eval(b, t(q))
+    u2, g2 = hp.hpfmm_eval(a, t(q))
+    assert torch.equal(u, u2) and torch.equal(g, g2)
