@@ -1580,8 +1580,9 @@ k_eval32m(const float2 *__restrict__ loc, const float *__restrict__ qsm, int rp,
           double *__restrict__ grad) {
   constexpr int NP = kMpW * kMpH;
   const float d = dg->d[H], invd = dg->invd[H];
-  __shared__ float2 spos[kMpCap];
-  __shared__ float4 sq[kMpCap * (RC / 4)];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  float2 *spos = reinterpret_cast<float2 *>(smem_raw);             // [kMpCap]
+  float4 *sq = reinterpret_cast<float4 *>(spos + kMpCap);          // [kMpCap][RC / 4]
   __shared__ int pst[NP + 1], pbeg[NP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nx = 1 << H;
@@ -1629,12 +1630,15 @@ k_eval32m(const float2 *__restrict__ loc, const float *__restrict__ qsm, int rp,
   const int ix = box_ix(leaf), iy = box_iy(leaf);
   const int px = ix - tx0 + 1, py = iy - ty0 + 1;  // patch coordinates of the leaf
   const int b0 = leaf_start[leaf], b1 = leaf_start[leaf + 1];
-  const int T = b1 - b0;
-  const int gs = T > 16 ? 32 : (T > 8 ? 16 : (T > 4 ? 8 : 4));
-  const int ng = 32 / gs, g = lane / gs, tli = lane % gs;
   const float c4 = (float)(0.69314718055994530942 / (4.0 * HP_PI));
   const float i2pi = (float)(1.0 / HP_TWO_PI);
-  for (int tb = b0; tb < b1; tb += gs) {
+  for (int tb = b0; tb < b1; tb += 32) {
+    // 32, 16, 8 or 4 targets a round, the groups of lanes taking interleaved
+    // sources: chosen for what is left, so that a leaf of 33 points does not
+    // take two rounds of 32
+    const int T = b1 - tb;
+    const int gs = T > 16 ? 32 : (T > 8 ? 16 : (T > 4 ? 8 : 4));
+    const int ng = 32 / gs, g = lane / gs, tli = lane % gs;
     const int i = tb + tli;
     const bool act = i < b1;
     const float2 me = act ? loc[i] : make_float2(0.f, 0.f);
@@ -1715,6 +1719,8 @@ k_eval32m(const float2 *__restrict__ loc, const float *__restrict__ qsm, int rp,
     }
   }
 }
+
+inline size_t eval32m_smem(int rc) { return kMpCap * (sizeof(float2) + sizeof(float) * (size_t)rc); }
 
 // Evaluation at separate targets (Example 2: field points that are not
 // sources, on y >= 0).  Targets stay in the caller's order and a warp takes
@@ -2065,6 +2071,8 @@ struct MultiWork {
   int nr, rp;
   void *qs, *qsm, *M, *A, *B;
 };
+// charge vectors per block of the multi-RHS S2M, and of the leaf kernel (16 when
+// there are more than 8: a pair's log2, reciprocal and loads serve twice as many)
 constexpr int kRhsChunk = 8;
 
 // separate targets: evaluate at (xt, yt) instead of at the sources
@@ -2371,10 +2379,11 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   }
   if constexpr (sizeof(R) == 4) {
     const float tau = pl->prec == HPFMM_MIXED ? (float)pl->tau_fp64 : 0.f;
-    k_eval32m<kRhsChunk><<<dim3(cdiv_u(pl->nleaf, kEvWarps), mw->rp / kRhsChunk), 32 * kEvWarps, 0,
-                           st>>>(pl->loc32, (const float *)mw->qsm, mw->rp, nr, pl->perm,
-                                 pl->leaf_start, H, dg, p, (const cf *)A, (const cf *)B, rs, pot,
-                                 grad);
+    const int rc = nr > kRhsChunk ? 2 * kRhsChunk : kRhsChunk;
+    auto *leaf = nr > kRhsChunk ? k_eval32m<2 * kRhsChunk> : k_eval32m<kRhsChunk>;
+    leaf<<<dim3(cdiv_u(pl->nleaf, kEvWarps), mw->rp / rc), 32 * kEvWarps, eval32m_smem(rc), st>>>(
+        pl->loc32, (const float *)mw->qsm, mw->rp, nr, pl->perm, pl->leaf_start, H, dg, p,
+        (const cf *)A, (const cf *)B, rs, pot, grad);
     pass_end(pl, st, PASS_EVAL, 1);
     pass_begin(pl, st, PASS_NEAR_MIRROR);
     auto *mir = nr > 32 ? k_mirror32m<64> : k_mirror32m<32>;
@@ -2415,7 +2424,13 @@ hpfmm_status fmm_set_smem_limits(int p) {
   HP_CUDA(prefer_shared(k_near32<2>));
   HP_CUDA(prefer_shared(k_near32<kTl>));
   HP_CUDA(prefer_shared(k_mirror32));
+<<<<<<< Updated upstream
   // (the highest order's: plans of several orders live beside one another)
+=======
+  HP_CUDA(cudaFuncSetAttribute(k_eval32m<2 * kRhsChunk>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)eval32m_smem(2 * kRhsChunk)));
+>>>>>>> Stashed changes
   HP_CUDA(cudaFuncSetAttribute(k_p2m64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)p2m64_smem(HPFMM_MAX_P)));
   HP_CUDA(cudaFuncSetAttribute(k_m2l_free<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64));
@@ -2461,7 +2476,10 @@ bool fmm_multi_supported(const hpfmm_plan *pl) {
          pl->p <= HPFMM_MAX_P;
 }
 
-int fmm_multi_rp(int nr) { return (nr + kRhsChunk - 1) / kRhsChunk * kRhsChunk; }
+int fmm_multi_rp(int nr) {
+  const int c = nr > kRhsChunk ? 2 * kRhsChunk : kRhsChunk;
+  return (nr + c - 1) / c * c;
+}
 
 hpfmm_status fmm_eval_targets(hpfmm_plan *pl, const double *q, const double *xt,
                               const double *yt, int64_t nt, const int64_t *blist,
