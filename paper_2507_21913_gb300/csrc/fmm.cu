@@ -2424,13 +2424,10 @@ hpfmm_status fmm_set_smem_limits(int p) {
   HP_CUDA(prefer_shared(k_near32<2>));
   HP_CUDA(prefer_shared(k_near32<kTl>));
   HP_CUDA(prefer_shared(k_mirror32));
-<<<<<<< Updated upstream
-  // (the highest order's: plans of several orders live beside one another)
-=======
   HP_CUDA(cudaFuncSetAttribute(k_eval32m<2 * kRhsChunk>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)eval32m_smem(2 * kRhsChunk)));
->>>>>>> Stashed changes
+  // (the highest order's: plans of several orders live beside one another)
   HP_CUDA(cudaFuncSetAttribute(k_p2m64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)p2m64_smem(HPFMM_MAX_P)));
   HP_CUDA(cudaFuncSetAttribute(k_m2l_free<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64));
