@@ -199,22 +199,27 @@ constexpr int kS2mGroup = 8;  // orders per thread of the single-precision S2M (
 // are sums of up to hundreds of terms of both signs, and their rounding error is
 // inherited by every far-field coefficient built from them.  (50021 points in
 // 1024 leaves with one lane an item: 16 blocks, 61 us.)
-constexpr int kS2mCap = 2048, kS2mThreads = 128;
+constexpr int kS2mLeaves = 64, kS2mCap = 2048, kS2mThreads = 128;
 
 __global__ void __launch_bounds__(kS2mThreads)
 k_s2m_tile(const float2 *__restrict__ loc, const float *__restrict__ qs,
-           const int *__restrict__ leaf_start, int H, int nlb, int S,
-           const DevGeom *__restrict__ dg, int p, cf *__restrict__ M, RhsStride rs) {
+           const int *__restrict__ leaf_start, int H, int nlb, const DevGeom *__restrict__ dg, int p,
+           cf *__restrict__ M, RhsStride rs) {
   constexpr int G = kS2mGroup;
   __shared__ float2 sp[kS2mCap];
   __shared__ float sq[kS2mCap];
+  __shared__ int ls[kS2mLeaves + 1], full[kS2mLeaves], nfull;
   pdl_trigger();  // the upward pass may be scheduled behind it
   const int P1 = p + 1, NB = (P1 + G - 1) / G;
   qs += blockIdx.y * rs.q;
   M += blockIdx.y * rs.m;
   const int nleaf = 1 << (2 * H);
   const int L0 = blockIdx.x * nlb, L1 = min(L0 + nlb, nleaf);
-  const int t0 = leaf_start[L0], t1 = leaf_start[L1];
+  const int nl = L1 - L0;
+  if (threadIdx.x == 0) nfull = 0;
+  for (int i = threadIdx.x; i <= nl; i += blockDim.x) ls[i] = leaf_start[L0 + i];
+  __syncthreads();
+  const int t0 = ls[0], t1 = ls[nl];
   const bool staged = t1 - t0 <= kS2mCap;
   if (staged) {
     for (int i = threadIdx.x; i < t1 - t0; i += blockDim.x) {
@@ -222,13 +227,25 @@ k_s2m_tile(const float2 *__restrict__ loc, const float *__restrict__ qs,
       sq[i] = qs[t0 + i];
     }
   }
+  // the leaves that hold points (on sources along a curve few of a tile's do);
+  // their order does not matter, the lanes a leaf follow from their number
+  const size_t m0 = ((size_t)level_offset(H) + L0) * P1;
+  for (int i = threadIdx.x; i < nl; i += blockDim.x)
+    if (ls[i + 1] > ls[i]) full[atomicAdd(&nfull, 1)] = i;
+  for (int e = threadIdx.x; e < nl * P1; e += blockDim.x) {
+    const int i = e / P1;
+    if (ls[i + 1] == ls[i]) M[m0 + e] = mk(0.f, 0.f);
+  }
   __syncthreads();
   const float invd = dg->invd[H];
-  const int nit = (L1 - L0) * NB, part = (int)threadIdx.x & (S - 1);
+  const int nit = nfull * NB;
+  int S = 1;
+  while (S < 16 && 2 * S * nit <= kS2mThreads) S *= 2;
+  const int part = (int)threadIdx.x & (S - 1);
   for (int it0 = 0; it0 < nit; it0 += kS2mThreads / S) {
     const int it = it0 + (int)threadIdx.x / S;
-    const int leaf = L0 + min(it, nit - 1) / NB, nb = it % NB, n0 = G * nb;
-    const int b0 = leaf_start[leaf], b1 = it < nit ? leaf_start[leaf + 1] : b0;
+    const int li = full[min(it, nit - 1) / NB], leaf = L0 + li, nb = it % NB, n0 = G * nb;
+    const int b0 = ls[li], b1 = it < nit ? ls[li + 1] : b0;
     // the compensated sums of the real and imaginary parts as paired FP32
     // additions (the same roundings as the scalar form)
     f2p acc[G], cmp[G];
@@ -2210,12 +2227,9 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
                                256, 0, fs>>>(pl->loc32, (const float *)mw->qsm, mw->rp, nr,
                                              pl->leaf_start, H, dg, p, (cf *)M, rs);
     else {
-      const int nlb = pl->nleaf >= 64 * 512 ? 64 : (pl->nleaf >= 16 * 256 ? 16 : 4);
-      const int items = nlb * ((P1 + kS2mGroup - 1) / kS2mGroup);
-      int S = 1;
-      while (S < 16 && 2 * S * items <= kS2mThreads) S *= 2;
+      const int nlb = pl->nleaf >= kS2mLeaves * 512 ? kS2mLeaves : (pl->nleaf >= 16 * 256 ? 16 : 4);
       k_s2m_tile<<<cdiv_u(pl->nleaf, nlb), kS2mThreads, 0, fs>>>(
-          pl->loc32, (const float *)qs, pl->leaf_start, H, nlb, S, dg, p, (cf *)M, rs);
+          pl->loc32, (const float *)qs, pl->leaf_start, H, nlb, dg, p, (cf *)M, rs);
     }
   }
   pass_end(pl, fs, PASS_P2M, 1);
