@@ -183,7 +183,6 @@ static void free_plan(hpfmm_plan *pl) {
   if (pl->ev_up) cudaEventDestroy(pl->ev_up);
   if (pl->ev_m2lh) cudaEventDestroy(pl->ev_m2lh);
   if (pl->ev_tree) cudaEventDestroy(pl->ev_tree);
-  if (pl->ev_geo) cudaEventDestroy(pl->ev_geo);
   if (pl->copy_stream) {
     cudaStreamSynchronize(pl->copy_stream);
     cudaStreamDestroy(pl->copy_stream);
@@ -269,14 +268,12 @@ static hpfmm_status rebuild(hpfmm_plan *pl, const double *x, const double *y, cu
   }
   hpfmm_status s = tree_build(pl, dx, dy, st);
   if (s == HPFMM_OK) {
-    // the geometry to the host and the reaction tables (they depend on the
-    // root square only) on the table stream, concurrent with what follows
-    // (ev_tree: recorded by tree_build after its last kernel)
+    // the reaction tables (they depend on the root square only) on the table
+    // stream, concurrent with what follows (ev_tree: recorded by tree_build
+    // after its last kernel).  The root square reaches the host by the build's
+    // own store to pinned memory: a copy on the table stream and its event
+    // came 10 us later.
     e = cudaStreamWaitEvent(pl->table_stream, pl->ev_tree, 0);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(pl->hgeo, pl->geo, 5 * sizeof(double), cudaMemcpyDeviceToHost,
-                          pl->table_stream);
-    if (e == cudaSuccess) e = cudaEventRecord(pl->ev_geo, pl->table_stream);
     if (e == cudaSuccess) s = tables_build(pl, pl->table_stream);
     if (e == cudaSuccess) e = cudaEventRecord(pl->ev_tables, pl->table_stream);
     if (e != cudaSuccess) {
@@ -286,9 +283,9 @@ static hpfmm_status rebuild(hpfmm_plan *pl, const double *x, const double *y, cu
     pl->tables_pending = true;
   }
   const bool sync = wait || pl->adaptive;
-  double hgeo[5] = {0, 0, 1, 0, 0};
+  double hgeo[4] = {0, 0, 1, 0};
   if (s == HPFMM_OK && sync) {
-    e = cudaEventSynchronize(pl->ev_geo);
+    e = cudaEventSynchronize(pl->ev_tree);
     if (e != cudaSuccess) {
       set_last_error("rebuild: %s", cudaGetErrorString(e));
       s = HPFMM_ECUDA;
@@ -316,7 +313,7 @@ static hpfmm_status rebuild(hpfmm_plan *pl, const double *x, const double *y, cu
 
 hpfmm_status plan_host_geometry(hpfmm_plan *pl) {
   if (!pl->geo_pending) return HPFMM_OK;
-  HP_CUDA(cudaEventSynchronize(pl->ev_geo));
+  HP_CUDA(cudaEventSynchronize(pl->ev_tree));
   pl->geo_pending = false;
   if (pl->hgeo[2] == 0.0) {
     pl->x0 = pl->hgeo[0];
@@ -527,7 +524,6 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_m2lh, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_up, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_tree, cudaEventDisableTiming);
-    if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_geo, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_tables, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming);
     if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&pl->ev_join, cudaEventDisableTiming);

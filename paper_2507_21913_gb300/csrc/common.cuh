@@ -407,11 +407,10 @@ struct hpfmm_plan {
   int64_t tlist_cap = 0;
   // the far-field chain of a split single-precision evaluation
   cudaStream_t side_stream = nullptr;
-  cudaEvent_t ev_geo = nullptr, ev_tables = nullptr;
-  // the geometry copy to the host and the reaction tables of a rebuild run on
-  // table_stream once the root square is known (ev_tree, recorded inside the
-  // tree build); the tables are joined into the evaluation's stream before
-  // the mirror M2L that reads them
+  cudaEvent_t ev_tables = nullptr;
+  // the reaction tables of a rebuild run on table_stream once the tree is built
+  // (ev_tree, after which the host copy of the geometry holds too); they are
+  // joined into the evaluation's stream before the mirror M2L that reads them
   cudaStream_t table_stream = nullptr;
   cudaEvent_t ev_tree = nullptr;
   // host-buffer calls: their copies on copy_stream, overlapping the tree
@@ -451,7 +450,7 @@ struct hpfmm_plan {
   unsigned *tree_ctr = nullptr;  // device: last-block counter of the tree build
   int *ctr = nullptr;     // device: last-block counters of the fused upward pass, one per RHS
   int async_update = 0;   // hpfmm_options.async_update
-  bool geo_pending = false;  // host copies x0 / side / qscale wait for ev_geo
+  bool geo_pending = false;  // host copies x0 / side / qscale wait for ev_tree
   void *tree_tmp = nullptr;  // tree-build temporaries, kept for the rebuilds of the plan
   int64_t tree_tmp_bytes = 0;
   int sms = 0;               // streaming multiprocessors of the plan's device

@@ -513,6 +513,7 @@ struct TreeBuild {
   double kabs;          // |kappa|: the I_n range check of an asynchronous rebuild
   int report;           // record invalid input / range in the status word
   double *geo;          // x0, side, invalid flag, 2^30 / side, largest bucket (int)
+  double *hgeo;         // the first four for the host (pinned memory)
   DevGeom *dg;          // level geometry
   uint64_t *keys;       // sorted keys
   int *leaf_start;      // nleaf + 1
@@ -657,7 +658,10 @@ k_tb_bbox(TreeBuild a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x < 4) a.geo[threadIdx.x] = sg[threadIdx.x];
+  if (threadIdx.x < 4) {
+    a.geo[threadIdx.x] = sg[threadIdx.x];
+    if (a.hgeo) a.hgeo[threadIdx.x] = sg[threadIdx.x];
+  }
   if (a.dg && threadIdx.x < 16) {
     const int l = threadIdx.x;
     const double d = ldexp(sg[1], -l);
@@ -1048,6 +1052,7 @@ hpfmm_status tree_build(hpfmm_plan *pl, const double *x, const double *y, cudaSt
   a.kabs = sqrt(pl->kre * pl->kre + pl->kim * pl->kim);
   a.report = pl->async_update;
   a.geo = pl->geo;
+  a.hgeo = pl->hgeo;
   a.dg = pl->dgeom;
   a.keys = pl->keys;
   a.leaf_start = pl->leaf_start;
@@ -1087,8 +1092,7 @@ hpfmm_status tree_build(hpfmm_plan *pl, const double *x, const double *y, cudaSt
     set_last_error("tree_build launch: %s", cudaGetErrorString(le));
     return HPFMM_ECUDA;
   }
-  // the reaction tables and the host copy of the root square start on the
-  // table stream once the build is done: run during the build, their
+  // the reaction tables start on the table stream once the build is done: run during the build, their
   // FP64-bound blocks slowed its short kernels by a third; after it they
   // share the SMs with the near field, which leaves the FP64 pipe idle
   if (pl->ev_tree) {
