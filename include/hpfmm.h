@@ -69,7 +69,9 @@ typedef enum {
   HPFMM_FP32 = 1,  /* P2P, M2L and expansions in single precision; translation
                       tables generated in double and rounded */
   HPFMM_MIXED = 2  /* as FP32, plus double precision for reaction P2P pairs
-                      with y_i + y_j < tau_fp64 (close to the boundary) */
+                      with y_i + y_j < tau_fp64 (close to the boundary; for
+                      |kappa| |s| <= 1/8 in float pairs good to 2^-36, the
+                      values being rounded to single precision either way) */
 } hpfmm_precision;
 
 typedef struct {

@@ -462,6 +462,8 @@ __device__ __forceinline__ void m2m_top(cpx<R> *Ms, int l0, int room, int P1,
     __syncthreads();
   }
   if (nb0 == chunk) return;
+  __threadfence();
+  __syncthreads();
   for (int e = threadIdx.x; e < 64 * P1; e += blockDim.x) {  // level 3, just written
     const int b = e / P1, m = e - b * P1;
     Ms[m2m_slot<R>(b, m, P1)] = ldcg_c(M + (size_t)level_offset(3) * P1 + e);

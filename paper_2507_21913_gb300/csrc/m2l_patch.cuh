@@ -61,11 +61,17 @@ namespace {
 // Where the accumulators would not fit (double precision beyond p = 25), the
 // output orders are taken in chunks.
 //
+// Measured (1e6 points, level 8, alone): single precision at p = 13 70 -> 51 us and
+// 66 M -> 22 M warp instructions (latency: 41 % of the issue slots), double
+// precision at p = 12 levels 2..8 2.87 -> 1.08 ms (the FP64 pipe).
+//
 // Two forms of the same kernel.  Wide: a warp takes 32 targets of one child type,
 // a lane each.  Narrow, for launches of few patches (below kWidePatches): a warp
 // takes 8 targets, four lanes each, every lane a quarter of the chunks of source
 // orders, their sums combined by shuffles: four times the blocks and a quarter
-// of each thread's chain, which is what bounds the small levels.  (A warp per
+// of each thread's chain, which is what bounds the small levels (single precision,
+// levels 2..7 at p = 13: 43 -> 37 us; double precision, level 5 at p = 24: 2.19 ->
+// 0.24 ms).  (A warp per
 // orbit instead ran seven different pieces of code once each and waited for
 // instructions.)
 constexpr int kPatchThreads = 128;
