@@ -8,7 +8,7 @@
 #include "common.cuh"
 #include "tc.cuh"
 
-hpfmm_status fmm_set_smem_limits(int p);
+hpfmm_status fmm_set_smem_limits();
 
 static thread_local char g_err[512] = "";
 
@@ -494,7 +494,7 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
     s = adaptive_alloc(pl);
     if (s != HPFMM_OK) { free_plan(pl); return s; }
   }
-  s = fmm_set_smem_limits(p);
+  s = fmm_set_smem_limits();
   if (s == HPFMM_OK) s = fmm_prepare();
   if (s == HPFMM_OK) s = adaptive_prepare();
   if (s == HPFMM_OK) s = near64_prepare();

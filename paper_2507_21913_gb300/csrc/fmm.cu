@@ -2419,8 +2419,20 @@ size_t fmm_shared_bytes_max(int p, bool fp64) {
   return (fp64 ? sizeof(cd) : sizeof(cf)) * (P1 * P1 + P1 * 33);
 }
 
-hpfmm_status fmm_set_smem_limits(int p) {
-  size_t s64 = fmm_shared_bytes_max(p, true), s32 = fmm_shared_bytes_max(p, false);
+hpfmm_status fmm_set_smem_limits() {
+  // once per device (none of the limits depends on the plan: about 40 calls)
+  static std::mutex mu;
+  static bool done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    set_last_error("fmm_set_smem_limits: no current device");
+    return HPFMM_ECUDA;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  if (done[dev]) return HPFMM_OK;
+  const size_t s64 = fmm_shared_bytes_max(HPFMM_MAX_P, true);
+  const size_t s32 = fmm_shared_bytes_max(HPFMM_MAX_P, false);
   // (the kernels of the split evaluation; those of the one-stream forms keep
   // the default split, with more L1)
   HP_CUDA(prefer_shared(k_gather_q<float>));
@@ -2468,6 +2480,7 @@ hpfmm_status fmm_set_smem_limits(int p) {
   HP_CUDA(cudaFuncSetAttribute(k_downward<float, true>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem));
   HP_CUDA(cudaFuncSetAttribute(k_m2l_free<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32));
+  done[dev] = true;
   return HPFMM_OK;
 }
 
