@@ -65,7 +65,9 @@ typedef enum {
 } hpfmm_status;
 
 typedef enum {
-  HPFMM_FP64 = 0,  /* every step in double precision (the plain path) */
+  HPFMM_FP64 = 0,  /* every step in double precision (the plain path); the
+                      free-space P2P pairs of orders up to 28 in 64-bit
+                      integers that hold no fewer bits */
   HPFMM_FP32 = 1,  /* P2P, M2L and expansions in single precision; translation
                       tables generated in double and rounded */
   HPFMM_MIXED = 2  /* as FP32, plus double precision for reaction P2P pairs

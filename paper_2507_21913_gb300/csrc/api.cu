@@ -463,8 +463,8 @@ extern "C" hpfmm_status hpfmm_create(const double *x, const double *y, int64_t n
     ALLOC(pl->mir_B, csz * 4 * (((size_t)1 << pl->H) - 1) * P1);
   }
   if (!f32) {
-    ALLOC(pl->fxy, sizeof(longlong2) * n);
-    ALLOC(pl->fq, sizeof(float2) * n);
+    ALLOC(pl->fxy, 16 * (size_t)n);
+    ALLOC(pl->fq, 16 * (size_t)n);
     ALLOC(pl->near64, 3 * sizeof(double) * n);
     ALLOC(pl->qexp, sizeof(int));
   }

@@ -437,9 +437,10 @@ struct hpfmm_plan {
   cudaEvent_t ev_up = nullptr;
   void *mir_A = nullptr, *mir_B = nullptr;
   float4 *near = nullptr;  // near-field sums per point (sorted order)
-  // double-precision plans (near64.cu): fixed-point coordinates and split
-  // charges of the free-space pairs, the sums (3 n doubles), the biased
-  // exponent of the largest charge (zeroed by the evaluation's last kernel)
+  // double-precision plans (near64.cu): fixed-point coordinates and charges of
+  // the free-space pairs, the sums (3 n doubles), twice the biased exponent of
+  // the largest charge or 1 where it is subnormal (zeroed by the evaluation's
+  // last kernel)
   void *fxy = nullptr, *fq = nullptr;
   double *near64 = nullptr;
   int *qexp = nullptr;

@@ -1,19 +1,11 @@
-// ff64.cuh -- double-precision pair arithmetic on the single-precision pipe.
-//
-// GB300 issues one FP64 warp instruction per ~19 cycles and SM (measured: 1.05
-// TFLOP/s against 78 in single precision), so an FP64 instruction costs as
-// much as 76 single-precision ones.  The free-space pairs of a
-// double-precision plan are therefore formed from integers and floats:
-//   - coordinates as 64-bit fixed point modulo 2^64, in units of 2^-61 of the
-//     power of two above the leaf side: the difference of two points of
-//     neighbouring leaves is one exact integer subtraction;
-//   - every further value as an unevaluated sum h + l of two floats (about 48
-//     bits), with the error-free sum and product of Dekker and Knuth;
-//   - sums over pairs as three floats, their two leading parts updated by
-//     error-free sums, so that a sum adds no error beyond the terms' own.
-// A term's relative error is a few 2^-49 (against the few 2^-53 of the FP64
-// expression); the sum over a leaf's neighbourhood, with 2^-70 or so of its
-// own, stays below the rounding that the double-precision far field adds.
+// ff64.cuh -- arithmetic of more than single precision on the single-precision
+// pipe: a value as an unevaluated sum h + l of two floats, about 48 bits, with the
+// error-free sum and product of Dekker and Knuth.  GB300 issues one FP64 warp
+// instruction per ~19 cycles and SM, so an FP64 instruction costs as much as 76
+// single-precision ones.  For values that are rounded to single precision in the
+// end (mirror_ff.cuh); the pairs of double-precision plans need more bits and take
+// integers (fix64.cuh).  The conversions from fixed point and the three-float sum
+// belong to the same arithmetic and are checked with it.
 //
 // The functions compile for the host as well (with the same roundings), so
 // that the arithmetic is checked on the CPU.

@@ -48,8 +48,9 @@ constexpr int kWarpsPerBlock = 4;
 // double-precision set-up arithmetic per thread: GB300's FP64 pipe is narrow).
 
 // --------------------------------------------------------------------------
-// gather the charges into tree order (qexp, when given, receives the biased
-// exponent of the largest charge, for the double-precision near field's split)
+// gather the charges into tree order (qexp, when given, receives twice the biased
+// exponent of the largest charge, or 1 where that is subnormal, for the
+// double-precision near field)
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm, int64_t n,
@@ -65,7 +66,7 @@ k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm, int64
       const double v = k < n ? q[perm[k]] : 0.0;
       if (k < n) qs[k] = v;
       const int e = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
-      const int m = __reduce_max_sync(0xffffffffu, e);
+      const int m = __reduce_max_sync(0xffffffffu, e > 0 ? 2 * e : (v != 0.0 ? 1 : 0));
       if ((threadIdx.x & 31) == 0) atomicMax(&smax, m);
       __syncthreads();
       if (threadIdx.x == 0 && smax > 0) atomicMax(qexp, smax);

@@ -8,36 +8,40 @@
 #include <mutex>
 
 #include "common.cuh"
-#include "ff64.cuh"
+#include "fix64.cuh"
 #include "pairs.cuh"
 #include "special.cuh"
 
 namespace {
 
-// ln table of ff_log, filled once per device
-__device__ ff g_log_tab[kFfLogN];
+// ln table of fx_pair, filled once per device
+__device__ int64_t g_log_tab[kFfLogN];
 
-// exponent of the power of two above the leaf side: the unit of the
-// fixed-point coordinates is 2^(kd - 60), so that differences between
-// neighbouring leaves stay below 2^61, and ff_from_fixed's results are in
-// units of 2^(kd - 23)
+// exponent of the power of two above the leaf side (fix64.cuh, kd)
 __device__ __forceinline__ int leaf_exponent(const DevGeom *dg, int H) {
   return (int)((__double_as_longlong(dg->side) >> 52) & 0x7ff) - 1022 - H;
 }
 
-// fixed-point coordinates and split charges of every point, in tree order.
-// The charges are scaled by the power of two of the largest (qexp, its biased
-// exponent, from the gather), so that their floats cannot leave the range.
+// a point's charge and the lowest 32 bits of its fixed-point coordinates, of
+// which the charge's drop (fix64.cuh) takes the last five of x
+struct __align__(16) FxRest {
+  int64_t q;
+  uint32_t ex, ey;
+  __device__ __forceinline__ int drop() const { return (int)(ex & 31u); }
+};
+
+// fixed-point coordinates and charges of every point, in tree order
 __global__ void __launch_bounds__(256)
 k_prep64(const double *__restrict__ xs, const double *__restrict__ ys,
          const double *__restrict__ qs, int64_t n, int H, const DevGeom *__restrict__ dg,
-         const int *__restrict__ qexp, longlong2 *__restrict__ fxy, float2 *__restrict__ fq) {
+         const int *__restrict__ qexp, ulonglong2 *__restrict__ fxy, FxRest *__restrict__ fq) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const int s = 60 - leaf_exponent(dg, H);
-  fxy[k] = make_longlong2(ff_fixed(xs[k], s), ff_fixed(ys[k], s));
-  const ff q = ff_split_scaled(qs[k], *qexp - 1023);
-  fq[k] = make_float2(q.h, q.l);
+  const fx96 x = fx_fixed(xs[k], s), y = fx_fixed(ys[k], s);
+  const FxCharge q = fx_charge(qs[k], *qexp >> 1);
+  fxy[k] = make_ulonglong2(x.v, y.v);
+  fq[k] = FxRest{q.bits, (x.e & ~31u) | (uint32_t)q.drop, y.e};
 }
 
 // The source ranges of a target's 3 x 3 neighbourhood, walked by a group of S
@@ -85,30 +89,33 @@ struct NearWalk {
 // (the coincident and the target's own point as in pair_free: only j = i is
 // left out).
 //
-// Bound by the single-precision issue slots: about 200 a pair (ff64.cuh), where
-// the FP64 expression took about 47 FP64 instructions = 3600 slots: a step of
-// 1e6 points at order 12 went from 28.4 to 4.65 ms (with the L2P taken out of
-// the leaf kernel and the far field beside it).  The lanes
-// of a warp are consecutive targets of two or three leaves; each walks its own
-// neighbourhood, so none idles for another's leaf, and the loads of one leaf's
-// lanes coincide.
+// Bound by the integer pipes, adder and multiplier at half the issue rate each:
+// about 215 warp instructions a pair with the walk, 100 of the one and 90 of the
+// other (fix64.cuh).  A step of 1e6 points at order 12, far field beside it, takes
+// 3.12 ms; 28.4 ms with FP64 pairs, 3.01 ms with pairs of floats, which held 48
+// bits and lost digits next to the axes.  The lanes of a warp are consecutive
+// targets of two or three leaves; each walks its own neighbourhood, so none idles
+// for another's leaf, and the loads of one leaf's lanes coincide.
 //
-// FF false: the pairs in FP64, for orders whose truncation error lies below the
-// pairs' 2^-48 and for trees of one level, whose sum is near field only; the
-// same where a charge is not finite (qexp at its top).
-template <bool FF>
-__global__ void __launch_bounds__(128)
+// FIX false: the pairs in FP64, for orders above 28 and for trees of one level,
+// whose sum is near field only; the same in either form for pairs closer than
+// fx_cut and where the largest charge is subnormal or not finite (qexp 1, or at
+// its top).
+template <bool FIX>
+__global__ void __launch_bounds__(128, 8)
 k_near64(const double *__restrict__ xs, const double *__restrict__ ys,
-         const double *__restrict__ qs, const longlong2 *__restrict__ fxy,
-         const float2 *__restrict__ fq, const uint64_t *__restrict__ keys,
+         const double *__restrict__ qs, const ulonglong2 *__restrict__ fxy,
+         const FxRest *__restrict__ fq, const uint64_t *__restrict__ keys,
          const int *__restrict__ leaf_start, int64_t n, int H, int S,
          const DevGeom *__restrict__ dg, const int *__restrict__ qexp,
          double *__restrict__ near) {
-  __shared__ ff tab[kFfLogN];
-  const int qe = FF ? *qexp : 0;
-  const bool fast = FF && qe != 0x7ff;
+  __shared__ int64_t tab[kFfLogN];
+  const int qe = FIX ? *qexp : 0;
+  const bool fast = FIX && qe != 1 && qe < 2 * 0x7ff;
+  const int kd = leaf_exponent(dg, H);
+  const FxScale sc = fx_scale(kd);
   if (fast) {
-    for (int e = threadIdx.x; e < kFfLogN; e += blockDim.x) tab[e] = g_log_tab[e];
+    for (int e = threadIdx.x; e < kFfLogN; e += blockDim.x) tab[e] = sc.tab(g_log_tab[e]);
     __syncthreads();
   }
   const int g = (int)(threadIdx.x & (S - 1)), per = (int)blockDim.x / S;
@@ -122,43 +129,31 @@ k_near64(const double *__restrict__ xs, const double *__restrict__ ys,
       NearWalk w;
       w.start(leaf_start, box_ix(leaf), box_iy(leaf), 1 << H, g);
       if (fast) {
-        // r^2 in units of 2^(2 kd - 46): the exponent's part of the log
-        const int ebias = 46 - 2 * leaf_exponent(dg, H);
-        const longlong2 me = fxy[i];
-        ff_sum3 sl{0.f, 0.f, 0.f}, sk{0.f, 0.f, 0.f}, sx{0.f, 0.f, 0.f}, sy{0.f, 0.f, 0.f};
+        const ulonglong2 mv = fxy[i];
+        const FxRest mr = fq[i];
+        FxSums a;
+        a.clear();
         for (; w.more(); w.step(S)) {
-          const longlong2 s = fxy[w.k];
-          const float2 qv = fq[w.k];
-          const int64_t DX = me.x - s.x, DY = me.y - s.y;
-          const int hx = (int)(DX >> 32), hy = (int)(DY >> 32);
-          if (((hx ^ (hx >> 31)) | (hy ^ (hy >> 31))) == 0) {
-            // closer than 2^-28 of the leaf side, where the fixed-point unit
-            // could show, or the target itself
+          const ulonglong2 v = fxy[w.k];
+          const FxRest r = fq[w.k];
+          const fx96 dx = fx_sub(fx96{mv.x, mr.ex}, fx96{v.x, r.ex});
+          const fx96 dy = fx_sub(fx96{mv.y, mr.ey}, fx96{v.y, r.ey});
+          const uint32_t reach = fx_reach(dx, dy);
+          if (reach < fx_cut(r.drop())) {  // or the target itself
             if (w.k != i) {
-              const double dx = xs[i] - xs[w.k], dy = ys[i] - ys[w.k];
-              PairAcc<double> a;
-              pair_free(a, dx, dy, qs[w.k]);
-              lf += a.lf;
-              gx += a.gfx;
-              gy += a.gfy;
+              PairAcc<double> d;
+              pair_free(d, xs[i] - xs[w.k], ys[i] - ys[w.k], qs[w.k]);
+              lf += d.lf;
+              gx += d.gfx;
+              gy += d.gfy;
             }
             continue;
           }
-          const ff dx = ff_from_fixed(DX), dy = ff_from_fixed(DY), q{qv.x, qv.y};
-          const ff r2 = ff_norm2(dx, dy);
-          const float c = ff_rcp_approx(r2.h);
-          float k;
-          sl.add(ff_prod(ff_log(r2, c, tab, ebias, k), q));
-          sk.add(ff_prod(ff{k, 0.f}, q));
-          const ff qw = ff_prod(ff_recip(r2, c), q);
-          sx.add(ff_prod(qw, dx));
-          sy.add(ff_prod(qw, dy));
+          fx_pair(a, dx, dy, reach, r.q, r.drop(), sc, tab);
         }
-        const double us = ldexp(1.0, qe - 1023);
-        const double ug = ldexp(1.0, qe - 1023 + 23 - leaf_exponent(dg, H));
-        lf += us * fma(0.69314718055994530942, sk.value(), sl.value());
-        gx += ug * sx.value();
-        gy += ug * sy.value();
+        lf += a.log_sum(qe >> 1, sc);
+        gx += a.gx(qe >> 1, kd);
+        gy += a.gy(qe >> 1, kd);
       } else {
         PairAcc<double> a;
         const double x = xs[i], y = ys[i];
@@ -261,8 +256,8 @@ hpfmm_status near64_prepare() {
   }
   std::lock_guard<std::mutex> lock(mu);
   if (done[dev]) return special_init_here();
-  static ff tab[kFfLogN];
-  ff_log_table(tab);
+  static int64_t tab[kFfLogN];
+  fx_log_table(tab);
   HP_CUDA(cudaMemcpyToSymbol(g_log_tab, tab, sizeof tab));
   HP_CUDA(prefer_shared(k_prep64));
   HP_CUDA(prefer_shared(k_near64<true>));
@@ -273,17 +268,15 @@ hpfmm_status near64_prepare() {
 }
 
 namespace {
-// The pairs' 2^-48 adds about 1e-15 to the relative error of the potential and
-// 4e-15 to the gradient's.  Up to order 28 that is below a tenth of the far
-// field's truncation (about 1.5e-14 and 6e-13 at 28, measured for 1000 to 60000
-// points); higher orders, and trees of one level, which have no free far
-// field, take FP64 pairs.
+// Up to order 28 the integer pairs; higher orders, and trees of one level, which
+// have no free far field, keep the FP64 pairs.
 bool near64_fast(const hpfmm_plan *pl) { return pl->p <= 28 && pl->H >= 2; }
 }  // namespace
 
-// Blocks per SM of the float-pair kernel, which loops over the targets: the far
-// field's kernels, bound by the FP64 pipe with few warps, find room beside them.
-constexpr int kNearBlocks = 5;
+// Blocks per SM of the integer kernel, which loops over the targets: the far
+// field's kernels, bound by the FP64 pipe with few warps, find room beside them
+// (the step above with 5, 6, 7, 8 blocks: 3.14, 3.12, 3.16, 3.27 ms).
+constexpr int kNearBlocks = 6;
 
 int near64_kernels(const hpfmm_plan *pl) { return near64_fast(pl) ? 2 : 1; }
 
@@ -296,11 +289,11 @@ hpfmm_status near64_launch(hpfmm_plan *pl, const double *qs, cudaStream_t st) {
   const unsigned nb = (unsigned)((n * S + 127) / 128);
   if (near64_fast(pl)) {
     k_prep64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pl->xs, pl->ys, qs, n, pl->H, pl->dgeom,
-                                                          pl->qexp, (longlong2 *)pl->fxy,
-                                                          (float2 *)pl->fq);
+                                                          pl->qexp, (ulonglong2 *)pl->fxy,
+                                                          (FxRest *)pl->fq);
     const unsigned most = (unsigned)(kNearBlocks * pl->sms);
-    k_near64<true><<<nb < most ? nb : most, 128, 0, st>>>(pl->xs, pl->ys, qs, (const longlong2 *)pl->fxy,
-                                       (const float2 *)pl->fq, pl->keys, pl->leaf_start, n, pl->H,
+    k_near64<true><<<nb < most ? nb : most, 128, 0, st>>>(pl->xs, pl->ys, qs, (const ulonglong2 *)pl->fxy,
+                                       (const FxRest *)pl->fq, pl->keys, pl->leaf_start, n, pl->H,
                                        S, pl->dgeom, pl->qexp, pl->near64);
   } else {
     k_near64<false><<<nb, 128, 0, st>>>(pl->xs, pl->ys, qs, nullptr, nullptr, pl->keys,
