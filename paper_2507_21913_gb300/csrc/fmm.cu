@@ -1303,9 +1303,10 @@ constexpr int kLsBytes = 80;       // tile leaf starts (kTl^2 + 1 ints), 16-byte
 // would cost close pairs their relative precision (an absolute error of
 // about 2^-25 d in every difference).  The target's own point is skipped by
 // index.  Lanes of one warp may belong to two or three leaves: they run the
-// same loops with their own bounds.  A 4 x 4 tile whose patch exceeds the buffer
-// is taken as four 2 x 2 tiles; a 2 x 2 tile's patch that still does reads from
-// global memory, leaf by leaf in leaf frames.
+// same loops with their own bounds.  A patch that exceeds the buffer is staged a
+// buffer at a time, the sums in global memory between (4000 points, 1800 of them
+// in one leaf: 9.2 ms an evaluation when each target read its sources from global
+// memory, 0.54 ms so).
 //
 // The buffer (26 KB) is kept small because the far-field kernels run beside
 // this one and need shared memory of their own on the same SMs: with 61 KB (one
@@ -1356,15 +1357,6 @@ __device__ __forceinline__ void pair_loop_self(const float4 *__restrict__ src,
   }
 }
 
-// the target (hi, lo) shifted by -c leaf sides, as hi + lo: |c d| >= |hi|
-// for c != 0, so the fast two-sum is exact (c = 0 leaves it unchanged)
-__device__ __forceinline__ void frame_shift(float hi, float lo, int c, float d, float dlo,
-                                            float &sh, float &sl) {
-  const float b = -(float)c * d;
-  sh = b + hi;
-  sl = (hi - (sh - b)) + (lo - (float)c * dlo);
-}
-
 // (h, l) + (oh, ol) as hi + lo: the two-sum of h and oh (exact for any
 // magnitudes), the low parts added
 __device__ __forceinline__ void add_hilo(float h, float l, float oh, float ol, float &sh,
@@ -1375,16 +1367,21 @@ __device__ __forceinline__ void add_hilo(float h, float l, float oh, float ol, f
   sl = (l + ol) + e;
 }
 
-// one tile of TL x TL leaves (fewer on a smaller tree) from leaf (tx0, ty0); false
-// when its patch exceeds the buffer and the caller takes it in quarters
 template <int TL>
-__device__ __forceinline__ bool near_tile(int tx0, int ty0, int nx, float d, float dlo,
-                                          const float2 *__restrict__ loc,
-                                          const float2 *__restrict__ loclo,
-                                          const double *__restrict__ q,
-                                          const int64_t *__restrict__ perm,
-                                          const int *__restrict__ leaf_start,
-                                          float4 *__restrict__ near) {
+__global__ void __launch_bounds__(kEvWarps * 32, 4)
+k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
+         const double *__restrict__ q, const int64_t *__restrict__ perm,
+         const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg,
+         float4 *__restrict__ near) {
+  // launched as a dependent of the tree build's last kernel; the charges are
+  // read in the caller's order through perm and rounded as the charge gather
+  // rounds them (bit-identical to the gathered copy), so that the gather runs
+  // beside this kernel instead of before it
+  pdl_wait();
+  const float d = dg->d[H], dlo = dg->dlo[H];
+  // a tile of TL x TL leaves (fewer on a smaller tree) from leaf (tx0, ty0)
+  const int nx = 1 << H, tps = nx >= TL ? nx / TL : 1;
+  const int tx0 = (blockIdx.x % tps) * TL, ty0 = (blockIdx.x / tps) * TL;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   int *ls = reinterpret_cast<int *>(smem_raw);         // [kTl^2 + 1] tile leaf starts
   float4 *src = reinterpret_cast<float4 *>(smem_raw + kLsBytes);  // [kTlCap] (hi, lo)
@@ -1431,106 +1428,87 @@ __device__ __forceinline__ bool near_tile(int tx0, int ty0, int nx, float d, flo
     offl[lane] = (float)(o - (double)oh);
   }
   __syncthreads();
-  const bool staged = pst[ps * ps] <= kTlCap;
-  if (!staged && TL > 2) return false;  // (the same for the whole block)
-  if (staged) {
-    for (int pi = warp; pi < ps * ps; pi += kEvWarps) {
-      const int b0 = pbeg[pi], cnt = pst[pi + 1] - pst[pi], o = pst[pi];
-      const float ohx = offh[pi % ps], olx = offl[pi % ps];
-      const float ohy = offh[pi / ps], oly = offl[pi / ps];
-      for (int j = lane; j < cnt; j += 32) {
-        const float2 v = loc[b0 + j], w = loclo[b0 + j];
-        float hx, lx, hy, ly;
-        add_hilo(v.x, w.x, ohx, olx, hx, lx);
-        add_hilo(v.y, w.y, ohy, oly, hy, ly);
-        src[o + j] = make_float4(hx, hy, lx, ly);
-        srcq[o + j] = fs_round(q[perm[b0 + j]]);
-      }
-    }
-  }
-  __syncthreads();
+  const int tot = pst[ps * ps];
   const int t0 = ls[0], t1 = ls[nlt];
-  for (int tb = t0 + 32 * warp; tb < t1; tb += 32 * kEvWarps) {
-    const int i = tb + lane;
-    const bool act = i < t1;
-    // the target's leaf: the last tile leaf whose start is <= i
+  // points j0 .. j1 - 1 of patch leaf pi to the buffer from o + j0 on
+  auto stage = [&](int pi, int j0, int j1, int o) {
+    const int b0 = pbeg[pi];
+    const float ohx = offh[pi % ps], olx = offl[pi % ps];
+    const float ohy = offh[pi / ps], oly = offl[pi / ps];
+    for (int j = j0 + lane; j < j1; j += 32) {
+      const float2 v = loc[b0 + j], w = loclo[b0 + j];
+      float hx, lx, hy, ly;
+      add_hilo(v.x, w.x, ohx, olx, hx, lx);
+      add_hilo(v.y, w.y, ohy, oly, hy, ly);
+      src[o + j] = make_float4(hx, hy, lx, ly);
+      srcq[o + j] = fs_round(q[perm[b0 + j]]);
+    }
+  };
+  // the tile leaf of target i: the last whose start is <= i
+  auto leaf_of = [&](int i) {
     int li = 0;
     for (int step = 8; step > 0; step >>= 1)
       if (li + step < nlt && ls[li + step] <= i) li += step;
-    const uint64_t leaf = L0 + li;
-    const int ix = box_ix(leaf), iy = box_iy(leaf);
-    const int px = ix - tx0 + 1, py = iy - ty0 + 1;
-    float lf = 0.f, gx = 0.f, gy = 0.f;
-    if (staged) {
-      const int kself = pst[py * ps + px] + (i - ls[li]);
-      float4 me = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (act) me = src[kself];
-      const f2p mh = f2_pack(me.x, me.y), ml = f2_pack(me.z, me.w);
-      f2p g = f2_pack(0.f, 0.f);
-#pragma unroll 1
-      for (int r = -1; r <= 1; ++r) {
-        const int pi = (py + r) * ps + px;
-        const int lo = pst[pi - 1];
-        const int hi = act ? pst[pi + 2] : lo;
-        if (r == 0) {
-          pair_loop_self(src, srcq, lo, hi, mh, ml, lf, g);
-        } else {
-          pair_loop(src, srcq, lo, hi, mh, ml, lf, g);
-        }
-      }
-      f2_unpack(g, gx, gy);
-    } else if (act) {
-      const float2 me = loc[i], ml = loclo[i];
-      for (int r = -1; r <= 1; ++r) {
-        float syh, syl;
-        frame_shift(me.y, ml.y, r, d, dlo, syh, syl);
-        for (int c = -1; c <= 1; ++c) {
-          const int mx = ix + c, my = iy + r;
-          if (mx < 0 || my < 0 || mx >= nx || my >= nx) continue;
-          const uint64_t sl = box_morton(mx, my);
-          const int s0 = leaf_start[sl], s1 = leaf_start[sl + 1];
-          float sxh, sxl;
-          frame_shift(me.x, ml.x, c, d, dlo, sxh, sxl);
-          for (int k = s0; k < s1; ++k) {
-            const float2 v = loc[k], w = loclo[k];
-            const float dx = (sxh - v.x) + (sxl - w.x), dy = (syh - v.y) + (syl - w.y);
-            const float r2 = fmaf(dx, dx, dy * dy);
-            if (!(r2 > 0.f)) continue;  // j = i, or a coincident point
-            const float qk = fs_round(q[perm[k]]);
-            const float qi = qk * fast_rcp(r2);
-            lf = fmaf(qk, fast_lg2(r2), lf);
-            gx = fmaf(qi, dx, gx);
-            gy = fmaf(qi, dy, gy);
-          }
-        }
-      }
-    }
-    if (act) near[i] = make_float4(lf, gx, gy, 0.f);
-  }
-  return true;
-}
-
-template <int TL>
-__global__ void __launch_bounds__(kEvWarps * 32, 4)
-k_near32(const float2 *__restrict__ loc, const float2 *__restrict__ loclo,
-         const double *__restrict__ q, const int64_t *__restrict__ perm,
-         const int *__restrict__ leaf_start, int H, const DevGeom *__restrict__ dg,
-         float4 *__restrict__ near) {
-  // launched as a dependent of the tree build's last kernel; the charges are
-  // read in the caller's order through perm and rounded as the charge gather
-  // rounds them (bit-identical to the gathered copy), so that the gather runs
-  // beside this kernel instead of before it
-  pdl_wait();
-  const float d = dg->d[H], dlo = dg->dlo[H];
-  const int nx = 1 << H, tps = nx >= TL ? nx / TL : 1;
-  const int tx0 = (blockIdx.x % tps) * TL, ty0 = (blockIdx.x / tps) * TL;
-  if (near_tile<TL>(tx0, ty0, nx, d, dlo, loc, loclo, q, perm, leaf_start, near)) return;
-  if constexpr (TL > 2) {
-    for (int s = 0; s < 4; ++s) {
-      const int x = tx0 + 2 * (s & 1), y = ty0 + 2 * (s >> 1);
+    return li;
+  };
+  if (tot > kTlCap) {  // (the same for the whole block)
+    for (int c0 = 0; c0 < tot; c0 += kTlCap) {
       __syncthreads();  // the staged points are replaced
-      if (x < nx && y < nx) near_tile<2>(x, y, nx, d, dlo, loc, loclo, q, perm, leaf_start, near);
+      for (int pi = warp; pi < ps * ps; pi += kEvWarps) {
+        const int o = pst[pi] - c0;
+        stage(pi, max(-o, 0), min(pst[pi + 1] - pst[pi], kTlCap - o), o);
+      }
+      __syncthreads();
+      for (int i = t0 + (int)threadIdx.x; i < t1; i += 32 * kEvWarps) {
+        const uint64_t leaf = L0 + leaf_of(i);
+        const int px = box_ix(leaf) - tx0 + 1, py = box_iy(leaf) - ty0 + 1;
+        const float2 v = loc[i], w = loclo[i];
+        float hx, lx, hy, ly;
+        add_hilo(v.x, w.x, offh[px], offl[px], hx, lx);
+        add_hilo(v.y, w.y, offh[py], offl[py], hy, ly);
+        const f2p mh = f2_pack(hx, hy), ml = f2_pack(lx, ly);
+        float4 sum = c0 > 0 ? near[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        f2p g = f2_pack(sum.y, sum.z);
+#pragma unroll 1
+        for (int r = -1; r <= 1; ++r) {
+          const int pi = (py + r) * ps + px;
+          pair_loop_self(src, srcq, max(pst[pi - 1] - c0, 0), min(pst[pi + 2] - c0, kTlCap), mh,
+                         ml, sum.x, g);
+        }
+        f2_unpack(g, sum.y, sum.z);
+        near[i] = sum;
+      }
     }
+    return;
+  }
+  for (int pi = warp; pi < ps * ps; pi += kEvWarps)
+    stage(pi, 0, pst[pi + 1] - pst[pi], pst[pi]);
+  __syncthreads();
+  for (int tb = t0 + 32 * warp; tb < t1; tb += 32 * kEvWarps) {
+    const int i = tb + lane;
+    const bool act = i < t1;
+    const int li = leaf_of(i);
+    const uint64_t leaf = L0 + li;
+    const int px = box_ix(leaf) - tx0 + 1, py = box_iy(leaf) - ty0 + 1;
+    const int kself = pst[py * ps + px] + (i - ls[li]);
+    float4 me = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (act) me = src[kself];
+    const f2p mh = f2_pack(me.x, me.y), ml = f2_pack(me.z, me.w);
+    float lf = 0.f, gx, gy;
+    f2p g = f2_pack(0.f, 0.f);
+#pragma unroll 1
+    for (int r = -1; r <= 1; ++r) {
+      const int pi = (py + r) * ps + px;
+      const int lo = pst[pi - 1];
+      const int hi = act ? pst[pi + 2] : lo;
+      if (r == 0) {
+        pair_loop_self(src, srcq, lo, hi, mh, ml, lf, g);
+      } else {
+        pair_loop(src, srcq, lo, hi, mh, ml, lf, g);
+      }
+    }
+    f2_unpack(g, gx, gy);
+    if (act) near[i] = make_float4(lf, gx, gy, 0.f);
   }
 }
 constexpr size_t kTpSmem = kLsBytes + (sizeof(float4) + sizeof(float)) * kTlCap +
