@@ -172,6 +172,8 @@ hpfmm_status hpfmm_update_points(hpfmm_plan *plan, const double *x, const double
  *   pot   : nrhs * n complex doubles (2 * nrhs * n doubles): u.
  *   grad  : NULL, or nrhs * n * 2 complex doubles: (du/dx_i, du/dy_i) per
  *           point (the field is minus this).
+ * Device pot and grad are aligned to a double, for single-precision plans on the
+ * uniform tree to 16 bytes (EINVAL otherwise).
  * Stream-ordered; returns without synchronising unless host buffers are
  * involved (then the results are in host memory when it returns).
  */

@@ -23,36 +23,35 @@
 
 namespace {
 
-__global__ void k_adj_split(const double2 *__restrict__ g, int64_t n, double *__restrict__ gr,
+__global__ void k_adj_split(const double *__restrict__ g, int64_t n, double *__restrict__ gr,
                             double *__restrict__ gi) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double2 v = g[i];
-  gr[i] = v.x;
-  gi[i] = v.y;
+  gr[i] = g[2 * i];
+  gi[i] = g[2 * i + 1];
 }
 
 // pot_*: complex u[Re g], u[Im g]; grad_*: complex (d/dx, d/dy) of the same and
-// of u[q]; all in caller (input) order
+// of u[q]; all in caller (input) order (g, gq and dxy are the caller's, aligned to
+// a double: read and written a double at a time)
 __global__ void k_adj_combine(int64_t n, const double *__restrict__ q,
-                              const double2 *__restrict__ g, const double2 *__restrict__ gq,
+                              const double *__restrict__ g, const double *__restrict__ gq,
                               const double2 *__restrict__ pot_r, const double2 *__restrict__ pot_i,
                               const double2 *__restrict__ grad_r,
                               const double2 *__restrict__ grad_i, double *__restrict__ dq,
-                              double2 *__restrict__ dxy) {
+                              double *__restrict__ dxy) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (dq) dq[i] = pot_r[i].x + pot_i[i].y;
   if (dxy) {
-    const double2 gv = g[i];
+    const double2 gv = make_double2(g[2 * i], g[2 * i + 1]);
     const double qi = q[i];
-    const double2 ax = gq[2 * i], ay = gq[2 * i + 1];
+    const double2 ax = make_double2(gq[4 * i], gq[4 * i + 1]);
+    const double2 ay = make_double2(gq[4 * i + 2], gq[4 * i + 3]);
     const double2 rx = grad_r[2 * i], ry = grad_r[2 * i + 1];
     const double2 ix = grad_i[2 * i], iy = grad_i[2 * i + 1];
-    double2 o;
-    o.x = gv.x * ax.x + gv.y * ax.y + qi * (rx.x + ix.y);
-    o.y = gv.x * ay.x + gv.y * ay.y + qi * (ry.x + iy.y);
-    dxy[i] = o;
+    dxy[2 * i] = gv.x * ax.x + gv.y * ax.y + qi * (rx.x + ix.y);
+    dxy[2 * i + 1] = gv.x * ay.x + gv.y * ay.y + qi * (ry.x + iy.y);
   }
 }
 
@@ -79,7 +78,7 @@ extern "C" hpfmm_status hpfmm_eval_adjoint(hpfmm_plan *pl, const double *q, cons
   double *grad_r = pot_i + 2 * n, *grad_i = grad_r + 4 * n;
   double *gq = grad_i + 4 * n, *pot_q = gq + 4 * n;
   const unsigned nb = (unsigned)((n + 255) / 256);
-  k_adj_split<<<nb, 256, 0, st>>>((const double2 *)g, n, gr, gi);
+  k_adj_split<<<nb, 256, 0, st>>>(g, n, gr, gi);
   HP_LAUNCH_CHECK();
   // transpose sums = forward sums with the real charge vectors Re g, Im g
   HP_TRY(fmm_eval(pl, gr, pot_r, dxy ? grad_r : nullptr, st));
@@ -88,10 +87,8 @@ extern "C" hpfmm_status hpfmm_eval_adjoint(hpfmm_plan *pl, const double *q, cons
     HP_TRY(fmm_eval(pl, q, pot_q, gq, st));
     grad_q = gq;
   }
-  k_adj_combine<<<nb, 256, 0, st>>>(n, q, (const double2 *)g, (const double2 *)grad_q,
-                                    (const double2 *)pot_r, (const double2 *)pot_i,
-                                    (const double2 *)grad_r, (const double2 *)grad_i, dq,
-                                    (double2 *)dxy);
+  k_adj_combine<<<nb, 256, 0, st>>>(n, q, g, grad_q, (const double2 *)pot_r, (const double2 *)pot_i,
+                                    (const double2 *)grad_r, (const double2 *)grad_i, dq, dxy);
   HP_LAUNCH_CHECK();
   return HPFMM_OK;
 }

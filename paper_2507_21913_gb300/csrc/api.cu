@@ -601,6 +601,7 @@ extern "C" hpfmm_status hpfmm_eval(hpfmm_plan *pl, const double *q, int nrhs, do
   const int64_t n = pl->n;
   bool qd = is_device_pointer(q), pd = is_device_pointer(pot);
   bool gd = !grad || is_device_pointer(grad);
+  HP_TRY(fmm_check_outputs(pl, pd ? pot : nullptr, gd ? grad : nullptr));
   const double *dq = q;
   double *dpot = pot, *dgrad = grad;
   if (!qd || !pd || !gd) HP_TRY(ensure_stage(pl, nrhs));

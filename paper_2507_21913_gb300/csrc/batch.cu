@@ -174,6 +174,7 @@ extern "C" hpfmm_status hpfmm_eval_batched(hpfmm_batch *b, const double *const *
         set_last_error("hpfmm_eval_batched: problem %d: arrays must be device memory", i);
         return HPFMM_EINVAL;
       }
+    HP_TRY(fmm_check_outputs(b->plans[i], pot[i], grad ? grad[i] : nullptr));
     if (b->plans[i]->timing) {
       set_last_error("hpfmm_eval_batched: problem %d has pass timing on", i);
       return HPFMM_EINVAL;

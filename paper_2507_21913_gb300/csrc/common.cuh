@@ -515,6 +515,8 @@ hpfmm_status adaptive_alloc(hpfmm_plan *pl);
 // device (a synchronous copy, so done at plan creation and never inside a
 // stream capture such as the batched graph)
 hpfmm_status fmm_prepare();
+// EINVAL where device outputs are not aligned as the plan's kernels store them
+hpfmm_status fmm_check_outputs(const hpfmm_plan *pl, const double *pot, const double *grad);
 hpfmm_status near64_prepare();
 hpfmm_status tables_prepare();
 // near field of a double-precision plan (near64.cu): the free-space pair sums

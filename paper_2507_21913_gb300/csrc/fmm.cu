@@ -756,20 +756,23 @@ k_downward(int H, int k, int p, const cpx<R> *__restrict__ Tl2l, cpx<R> *__restr
       gx.x = fma(-i2pi, fx, gx.x);
       gy.x = fma(-i2pi, fy, gy.x);
       const int64_t o = ev.perm[i];
-      double2 *po = reinterpret_cast<double2 *>(ev.pot) + o;
-      double2 *go = reinterpret_cast<double2 *>(ev.grad) + 2 * o;
+      // (a double at a time: the caller's complex arrays need no more than a
+      // double's alignment)
+      double *po = ev.pot + 2 * o, *go = ev.grad + 4 * o;
       if (iy == 0) {  // bottom row: image/reaction sums already there
-        const double2 pm = *po;
-        u = u + mk(pm.x, pm.y);
+        u = u + mk(po[0], po[1]);
         if (ev.grad) {
-          gx = gx + mk(go[0].x, go[0].y);
-          gy = gy + mk(go[1].x, go[1].y);
+          gx = gx + mk(go[0], go[1]);
+          gy = gy + mk(go[2], go[3]);
         }
       }
-      *po = make_double2(u.x, u.y);
+      po[0] = u.x;
+      po[1] = u.y;
       if (ev.grad) {
-        go[0] = make_double2(gx.x, gx.y);
-        go[1] = make_double2(gy.x, gy.y);
+        go[0] = gx.x;
+        go[1] = gx.y;
+        go[2] = gy.x;
+        go[3] = gy.y;
       }
     }
   } else if constexpr (EVAL) {
@@ -2466,6 +2469,14 @@ hpfmm_status fmm_set_smem_limits() {
 hpfmm_status fmm_prepare() {
   HP_TRY(mirror_tables_here());
   return special_init_here();
+}
+
+hpfmm_status fmm_check_outputs(const hpfmm_plan *pl, const double *pot, const double *grad) {
+  if (pl->prec == HPFMM_FP64 || pl->adaptive) return HPFMM_OK;  // written a double at a time
+  if ((((uintptr_t)pot | (uintptr_t)grad) & 15) == 0) return HPFMM_OK;
+  set_last_error("pot and grad of a single-precision plan on the uniform tree must be aligned to "
+                 "16 bytes");
+  return HPFMM_EINVAL;
 }
 
 hpfmm_status fmm_eval(hpfmm_plan *pl, const double *q, double *pot, double *grad,

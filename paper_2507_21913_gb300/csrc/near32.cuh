@@ -188,27 +188,24 @@ struct MirrorAcc {
 #pragma unroll
       for (int o = G / 2; o > 0; o >>= 1) v[e] += __shfl_xor_sync(mask, v[e], o);
   }
-  // to the outputs of point o: assigned, or added to what is there
+  // to the outputs of point o: assigned, or added to what is there (a double at a
+  // time: the caller's complex arrays need no more than a double's alignment)
   __device__ __forceinline__ void put(double *pot, double *grad, int64_t o, bool assign) const {
-    double2 *po = reinterpret_cast<double2 *>(pot) + o;
-    double2 *go = reinterpret_cast<double2 *>(grad) + 2 * o;
-    double2 a = make_double2(f2d(v[0]), f2d(v[1]));
-    double2 b = make_double2(f2d(v[2]), f2d(v[3])), c = make_double2(f2d(v[4]), f2d(v[5]));
+    double *po = pot + 2 * o, *go = grad + 4 * o;
+    double a[6];
+#pragma unroll
+    for (int e = 0; e < 6; ++e) a[e] = f2d(v[e]);
     if (!assign) {
-      const double2 t = *po;
-      a.x += t.x;
-      a.y += t.y;
+      a[0] += po[0];
+      a[1] += po[1];
     }
-    *po = a;
+    po[0] = a[0];
+    po[1] = a[1];
     if (!grad) return;
-    if (!assign) {
-      const double2 t = go[0], u = go[1];
-      b.x += t.x;
-      b.y += t.y;
-      c.x += u.x;
-      c.y += u.y;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (!assign) a[2 + e] += go[e];
+      go[e] = a[2 + e];
     }
-    go[0] = b;
-    go[1] = c;
   }
 };
