@@ -42,8 +42,7 @@ constexpr int kRecip = 512;
 static __constant__ double c_recip[kRecip];
 // Coefficients of the J_0 and J_1 power series (j01_arg), c_ser[0][k] = 1/(k k!)
 // and c_ser[1][k] = 1/((k-1) k!), and the terms they need: c_nser[i] for
-// |P| <= (i + 1) / 4 (a^N / N! <= 1e-17 max(1, a^2), well below the rounding of
-// the sum).
+// |P| <= (i + 1) / 4 (a^N / N! <= 1e-18, well below the rounding of the sum).
 constexpr int kSer = 64, kNser = 16;
 static __constant__ double c_ser[2][kSer];
 static __constant__ int c_nser[kNser];
@@ -232,8 +231,9 @@ __device__ __forceinline__ void j01_arg(cd P, double P2, float a, double lr, dou
                                         cd &J0, cd &J1) {
   const bool big = P2 >= 1.0;
   if (a <= 0.5f || (a <= 4.0f && (double)a - P.x <= 1.5)) {
-    // the lanes take one term count: the coefficients are read uniformly
-    const int N = __reduce_max_sync(__activemask(), c_nser[min((int)(4.0f * a), kNser - 1)]);
+    // each lane its own term count, so that a pair's value does not depend on the
+    // pairs beside it
+    const int N = c_nser[min((int)(4.0f * a), kNser - 1)];
     const double r = P.x + P.x;
     double b1 = 0.0, b2 = 0.0;
     if (!big) {
