@@ -444,6 +444,7 @@ struct hpfmm_plan {
   void *fxy = nullptr, *fq = nullptr;
   double *near64 = nullptr;
   int *qexp = nullptr;
+  bool qexp_clear = true;  // false while an evaluation has been issued in part
   double *hgeo = nullptr;  // pinned host copy of geo, written by the tree build
   int *status = nullptr;  // device status word
   double *geo = nullptr;  // device: x0, side, invalid flag, 2^30/side, largest leaf (int)

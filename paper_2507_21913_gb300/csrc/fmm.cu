@@ -2141,6 +2141,12 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
     HP_CUDA(cudaStreamWaitEvent(pl->side_stream, pl->ev_fork, 0));
     fs = pl->side_stream;
   }
+  if (split && sizeof(R) == 8) {
+    // cleared by the last evaluation's downward pass, unless that one failed
+    // before it (on this stream: after the charges that one gathered)
+    if (!pl->qexp_clear) HP_CUDA(cudaMemsetAsync(pl->qexp, 0, sizeof(int), fs));
+    pl->qexp_clear = false;
+  }
   // the charges in tree order: first on the far-field chain when split (the
   // near field reads them through perm itself)
   pass_begin(pl, fs, PASS_GATHER);
@@ -2343,6 +2349,7 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
         mirror_apart ? (const cpx<R> *)pl->mir_B : nullptr);
     pass_end(pl, st, PASS_L2L, 1);
     HP_LAUNCH_CHECK();
+    if (sizeof(R) == 8) pl->qexp_clear = true;
     return HPFMM_OK;
   }
   pass_begin(pl, fs, PASS_L2L);
