@@ -203,7 +203,7 @@ static void free_plan(hpfmm_plan *pl) {
   void *bufs[] = {pl->xs, pl->ys, pl->perm, pl->keys, pl->leaf_start, pl->loc32, pl->yabs, pl->t_m2m,
                   pl->t_l2l, pl->t_m2l, pl->t_refl, pl->t_rlog, pl->t_rlog0, pl->qs, pl->M,
                   pl->A, pl->B, pl->out_pot, pl->out_grad, pl->in_q, pl->status,
-                  pl->t_binom, pl->geo, pl->t_m2l_pad, pl->adj, pl->mq, pl->mqsm,
+                  pl->t_binom, pl->geo, pl->t_m2l_pad, pl->adj, pl->mqsm,
                   pl->mM, pl->mA, pl->mB, pl->tflag, pl->tlist, pl->t_m2l_tc,
                   pl->ab_key, pl->ab_lo, pl->ab_hi, pl->ab_parent, pl->ab_lvl, pl->ab_child,
                   pl->ab_cut, pl->ab_off, pl->ab_idx, pl->ab_lev, pl->ab_btot, pl->ab_lrank,
@@ -575,14 +575,13 @@ constexpr int kMultiMax = 64;
 
 static hpfmm_status ensure_multi(hpfmm_plan *pl, int nr) {
   if (pl->mcap >= nr) return HPFMM_OK;
-  void **bufs[] = {&pl->mq, &pl->mqsm, &pl->mM, &pl->mA, &pl->mB};
+  void **bufs[] = {&pl->mqsm, &pl->mM, &pl->mA, &pl->mB};
   for (void **b : bufs) {
     if (*b) cudaFree(*b);
     *b = nullptr;
   }
   pl->mcap = 0;
   const size_t n = (size_t)pl->n, ncoef = (size_t)pl->nbox * (pl->p + 1);
-  HP_TRY(plan_dalloc(pl, &pl->mq, sizeof(float) * n * nr));
   HP_TRY(plan_dalloc(pl, &pl->mqsm, sizeof(float) * n * fmm_multi_rp(nr)));
   HP_TRY(plan_dalloc(pl, &pl->mM, 2 * sizeof(float) * ncoef * nr));
   HP_TRY(plan_dalloc(pl, &pl->mA, 2 * sizeof(float) * ncoef * nr));
@@ -627,8 +626,8 @@ extern "C" hpfmm_status hpfmm_eval(hpfmm_plan *pl, const double *q, int nrhs, do
     for (int r0 = 0; r0 < nrhs; r0 += chunk) {
       const int nr = nrhs - r0 < chunk ? nrhs - r0 : chunk;
       HP_TRY(fmm_eval_multi(pl, dq + (size_t)r0 * n, nr, dpot + (size_t)2 * r0 * n,
-                            dgrad ? dgrad + (size_t)4 * r0 * n : nullptr, pl->mq, pl->mqsm,
-                            pl->mM, pl->mA, pl->mB, st));
+                            dgrad ? dgrad + (size_t)4 * r0 * n : nullptr, pl->mqsm, pl->mM,
+                            pl->mA, pl->mB, st));
     }
   } else {
     for (int r = 0; r < nrhs; ++r) {

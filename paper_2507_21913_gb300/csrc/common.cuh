@@ -398,7 +398,7 @@ struct hpfmm_plan {
   int64_t stage_rhs = 0;
   double *adj = nullptr;  // adjoint workspace (20 n doubles), allocated on first use
   // multi-RHS workspace (single precision), for up to mcap charge vectors at once
-  void *mq = nullptr, *mqsm = nullptr, *mM = nullptr, *mA = nullptr, *mB = nullptr;
+  void *mqsm = nullptr, *mM = nullptr, *mA = nullptr, *mB = nullptr;
   int mcap = 0;
   // hpfmm_eval_targets: validation flag and bottom-row target count (int[2]);
   // the list of targets in the bottom leaf row (single-precision plans)
@@ -532,7 +532,7 @@ hpfmm_status fmm_eval_targets(hpfmm_plan *pl, const double *q, const double *xt,
                               int64_t nbottom, double *pot, double *grad, cudaStream_t st);
 int fmm_multi_rp(int nr);
 hpfmm_status fmm_eval_multi(hpfmm_plan *pl, const double *q, int nr, double *pot, double *grad,
-                            void *qs, void *qsm, void *M, void *A, void *B, cudaStream_t st);
+                            void *qsm, void *M, void *A, void *B, cudaStream_t st);
 bool is_device_pointer(const void *p);
 hpfmm_status plan_dalloc(hpfmm_plan *pl, void **p, size_t bytes);
 // host copies of the root square (x0, side, qscale) of the current tree: waits

@@ -81,15 +81,14 @@ k_gather_q(const double *__restrict__ q, const int64_t *__restrict__ perm, int64
     qs[k] = qd;
 }
 
-// the same for nr charge vectors of a multi-RHS evaluation: qs[r n + k] and the
-// point-major copy qsm[k rp + r].  A warp takes 32 points, a vector at a time,
-// and turns them around in shared memory, so that both copies are written in
-// whole rows (one thread per value wrote qsm 4 bytes a sector: 360 us for 64
-// vectors of 500000).
+// the same for nr charge vectors of a multi-RHS evaluation, point-major: qsm[k rp + r].
+// A warp takes 32 points, a vector at a time, and turns them around in shared
+// memory, so that they are written in whole rows (one thread per value wrote qsm 4
+// bytes a sector: 360 us for 64 vectors of 500000).
 constexpr int kGmWarps = 4, kGmR = 32;  // vectors per block
 __global__ void __launch_bounds__(32 * kGmWarps)
 k_gather_multi(const double *__restrict__ q, const int64_t *__restrict__ perm, int64_t n, int nr,
-               float *__restrict__ qs, float *__restrict__ qsm, int rp) {
+               float *__restrict__ qsm, int rp) {
   pdl_wait();  // launched as a dependent of the tree build's last kernel
   pdl_trigger();
   __shared__ float tile[32][kGmR + 1];
@@ -100,12 +99,7 @@ k_gather_multi(const double *__restrict__ q, const int64_t *__restrict__ perm, i
 #pragma unroll
   for (int j = warp; j < kGmR; j += kGmWarps) {
     const int r = r0 + j;
-    float v = 0.0f;
-    if (r < nr && k < n) {
-      v = fs_round(q[(size_t)r * n + o]);
-      qs[(size_t)r * n + k] = v;
-    }
-    tile[lane][j] = v;
+    tile[lane][j] = r < nr && k < n ? fs_round(q[(size_t)r * n + o]) : 0.0f;
   }
   __syncthreads();
   if (r0 + lane < rp)
@@ -2070,7 +2064,7 @@ inline unsigned cdiv_u(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b
 // up to the leaf kernel's RHS chunk; arrays of the evaluation's real type
 struct MultiWork {
   int nr, rp;
-  void *qs, *qsm, *M, *A, *B;
+  void *qsm, *M, *A, *B;
 };
 // charge vectors per block of the multi-RHS S2M, and of the leaf kernel (16 when
 // there are more than 8: a pair's log2, reciprocal and loads serve twice as many)
@@ -2102,7 +2096,7 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   const cpx<R> *Treact = tab(pl->t_refl, (size_t)H * 42 * m2);
   const cd *logs = (const cd *)pl->t_rlog0;
   const int nr = mw ? mw->nr : 1;
-  R *qs = (R *)(mw ? mw->qs : pl->qs);
+  R *qs = (R *)pl->qs;  // (many charge vectors: mw->qsm)
   cpx<R> *M = (cpx<R> *)(mw ? mw->M : pl->M), *A = (cpx<R> *)(mw ? mw->A : pl->A);
   cpx<R> *B = (cpx<R> *)(mw ? mw->B : pl->B);
   const RhsStride rs{n, pl->nbox * (int64_t)P1, 2 * n};
@@ -2154,8 +2148,8 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
     k_gather_q<R><<<dim3(cdiv_u(n, 256)), 256, 0, fs>>>(q, pl->perm, n, qs, pl->qexp);
   else if (mw)
     HP_CUDA(launch_dependent(k_gather_multi, dim3(cdiv_u(n, 32), cdiv_u(mw->rp, kGmR)),
-                             dim3(32 * kGmWarps), 0, st, q, pl->perm, n, nr, (float *)qs,
-                             (float *)mw->qsm, mw->rp));
+                             dim3(32 * kGmWarps), 0, st, q, pl->perm, n, nr, (float *)mw->qsm,
+                             mw->rp));
   else
     HP_CUDA(launch_dependent(k_gather_q<R>, dim3(cdiv_u(n, 256)), dim3(256), 0, st, q, pl->perm, n,
                              qs, (int *)nullptr));
@@ -2514,12 +2508,12 @@ hpfmm_status fmm_eval_targets(hpfmm_plan *pl, const double *q, const double *xt,
 }
 
 hpfmm_status fmm_eval_multi(hpfmm_plan *pl, const double *q, int nr, double *pot, double *grad,
-                            void *qs, void *qsm, void *M, void *A, void *B, cudaStream_t st) {
+                            void *qsm, void *M, void *A, void *B, cudaStream_t st) {
   HP_TRY(special_init_here());
   if (!fmm_multi_supported(pl)) {
     set_last_error("multi-RHS passes need single precision, >= 2 levels and p >= 2");
     return HPFMM_EUNSUPPORTED;
   }
-  const MultiWork mw{nr, fmm_multi_rp(nr), qs, qsm, M, A, B};
+  const MultiWork mw{nr, fmm_multi_rp(nr), qsm, M, A, B};
   return run_passes<float>(pl, q, pot, grad, st, &mw);
 }
