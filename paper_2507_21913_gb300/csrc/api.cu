@@ -570,9 +570,6 @@ static hpfmm_status ensure_stage(hpfmm_plan *pl, int nrhs) {
   return HPFMM_OK;
 }
 
-// charge vectors per multi-RHS pass set
-constexpr int kMultiMax = 64;
-
 static hpfmm_status ensure_multi(hpfmm_plan *pl, int nr) {
   if (pl->mcap >= nr) return HPFMM_OK;
   void **bufs[] = {&pl->mqsm, &pl->mM, &pl->mA, &pl->mB};

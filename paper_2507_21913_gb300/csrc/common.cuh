@@ -530,6 +530,7 @@ hpfmm_status adaptive_prepare();
 hpfmm_status fmm_eval_targets(hpfmm_plan *pl, const double *q, const double *xt,
                               const double *yt, int64_t nt, const int64_t *blist,
                               int64_t nbottom, double *pot, double *grad, cudaStream_t st);
+constexpr int kMultiMax = 64;  // charge vectors per multi-RHS pass set
 int fmm_multi_rp(int nr);
 hpfmm_status fmm_eval_multi(hpfmm_plan *pl, const double *q, int nr, double *pot, double *grad,
                             void *qsm, void *M, void *A, void *B, cudaStream_t st);

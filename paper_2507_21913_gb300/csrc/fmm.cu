@@ -1952,7 +1952,8 @@ k_mirror32(const float2 *__restrict__ loc, const float *__restrict__ yabs,
 // through shared memory to lanes that take one charge vector each (RB = 32 or 64
 // in all; charges point-major, qsm[k * rp + r], one coalesced row a source).  A
 // pair's 130 instructions serve all vectors, which then take six products each.
-constexpr int kMirmWarps = 4;
+constexpr int kMirmWarps = 4, kMirmMost = 64;
+static_assert(kMultiMax <= kMirmMost, "k_mirror32m takes one lane slot a vector");
 template <int RB>
 __global__ void __launch_bounds__(32 * kMirmWarps)
 k_mirror32m(const float2 *__restrict__ loc, const float *__restrict__ yabs,
@@ -2385,7 +2386,7 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
         (const cf *)A, (const cf *)B, rs, pot, grad);
     pass_end(pl, st, PASS_EVAL, 1);
     pass_begin(pl, st, PASS_NEAR_MIRROR);
-    auto *mir = nr > 32 ? k_mirror32m<64> : k_mirror32m<32>;
+    auto *mir = nr > 32 ? k_mirror32m<kMirmMost> : k_mirror32m<32>;
     mir<<<dim3((unsigned)(1 << H), 1, kMirSplit), 32 * kMirmWarps, 0, st>>>(
         pl->loc32, pl->yabs, (const float *)mw->qsm, mw->rp, nr, pl->perm, pl->leaf_start, H, dg,
         kappa_log(pl->kre, pl->kim), tau, pot, grad, rs);
@@ -2510,6 +2511,10 @@ hpfmm_status fmm_eval_targets(hpfmm_plan *pl, const double *q, const double *xt,
 hpfmm_status fmm_eval_multi(hpfmm_plan *pl, const double *q, int nr, double *pot, double *grad,
                             void *qsm, void *M, void *A, void *B, cudaStream_t st) {
   HP_TRY(special_init_here());
+  if (nr > kMultiMax) {
+    set_last_error("multi-RHS passes take at most %d charge vectors at a time", kMultiMax);
+    return HPFMM_EINVAL;
+  }
   if (!fmm_multi_supported(pl)) {
     set_last_error("multi-RHS passes need single precision, >= 2 levels and p >= 2");
     return HPFMM_EUNSUPPORTED;
