@@ -126,18 +126,22 @@ __device__ __forceinline__ void exp_sum_f(cf P, float P2, cf &E, cf &S) {
 
 // Single precision where the series is accurate (|P| <= 1) and the pair is not
 // below tau, else float pairs (|P| <= 1/8, s2 well inside the float range; 4e6
-// clustered points in MIXED mode: 7.87 ms a step with FP64, 5.45 so) or double.  X the difference of the x, Y the sum of the y.  ln
-// and reciprocal of X^2 + Y^2 serve the image and both reaction terms, and for
-// real kappa the arguments P+- are conjugate, J_n(conj P) = conj J_n(P) + 2 pi i
-// conj(P)^n e^{-conj P}: about 130 instructions a pair (two complex series, four
-// divisions and the accumulation for one charge took about 450).
+// clustered points in MIXED mode: 7.87 ms a step with FP64, 5.45 so) or double.  X
+// the difference of the x, Y the sum of the y.  The reciprocal of X^2 + Y^2 serves the
+// image and both reaction terms, and for real kappa the arguments P+- are conjugate,
+// J_n(conj P) = conj J_n(P) + 2 pi i conj(P)^n e^{-conj P}: about 130 instructions a
+// pair (two complex series, four divisions and the accumulation for one charge took
+// about 450).
 __device__ __forceinline__ MirrorVal mirror_value(float X, float Y, const KappaF &kf,
                                                   const KappaLog &K, float tau) {
   const float s2 = fmaf(X, X, Y * Y), P2 = kf.a2 * s2;
   if (!(P2 <= 1.0f && Y >= tau))
     return P2 <= 0.0156f && s2 >= 1e-24f ? mirror_value_ff(K, X, Y) : mirror_value_d(K, X, Y);
   const float ln = 0.693147180559945f * fast_lg2(s2), inv = fast_rcp(s2);
-  const float lr = fmaf(0.5f, ln, kf.lk), th = atan2f(X, Y);
+  // (ln |P| of its own: as ln |s| + ln |kappa| it loses what the two cancel; that for
+  // P2 near the end of the float range)
+  const float lr = P2 > 1e-30f ? 0.346573590279973f * fast_lg2(P2) : fmaf(0.5f, ln, kf.lk);
+  const float th = atan2f(X, Y);
   const float g = -(float)HP_EULER_GAMMA - lr, pi = (float)HP_PI;
   const cf Pp = kf.kappa * mk(Y, -X), Pm = kf.kappa * mk(Y, X);
   cf Ep, Sp, Em, Sm;
