@@ -41,8 +41,6 @@
 
 namespace {
 
-constexpr int kWarpsPerBlock = 4;
-
 // Box side, its reciprocal and log per level come from the plan's DevGeom
 // record, written on the device by the tree build (no kernel repeats
 // double-precision set-up arithmetic per thread: GB300's FP64 pipe is narrow).
@@ -2110,8 +2108,8 @@ hpfmm_status run_passes(hpfmm_plan *pl, const double *q, double *pot, double *gr
   // one RHS, the sources as targets ("split"): the free-space near field
   // needs only the sorted points and charges, so it runs on this stream while
   // the plan's side stream runs the far-field passes; L2P joins them.  In
-  // double precision the near field takes the single-precision pipe (near64.cu)
-  // and the far field the FP64 pipe, so the two overlap.
+  // double precision the near field takes the integer pipes (near64.cu) and
+  // the far field the FP64 pipe, so the two overlap.
   const bool split = !mw && !tw;
   if (split && !((sizeof(R) == 4 ? (void *)pl->near : (void *)pl->near64) && pl->side_stream &&
                  pl->m2l_stream && pl->ev_fork && pl->ev_join && pl->ev_gather && pl->ev_m2lh)) {

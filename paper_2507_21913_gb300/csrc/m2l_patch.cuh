@@ -61,9 +61,9 @@ namespace {
 // Where the accumulators would not fit (double precision beyond p = 25), the
 // output orders are taken in chunks.
 //
-// Measured (1e6 points, level 8, alone): single precision at p = 13 70 -> 51 us and
-// 66 M -> 22 M warp instructions (latency: 41 % of the issue slots), double
-// precision at p = 12 levels 2..8 2.87 -> 1.08 ms (the FP64 pipe).
+// Measured (1e6 points, level 8, alone): single precision at p = 13 70 -> 45 us and
+// 66 M -> 21 M warp instructions (latency: 43 % of the issue slots), double
+// precision at p = 12 levels 2..8 2.87 -> 1.07 ms (the FP64 pipe).
 //
 // Two forms of the same kernel.  Wide: a warp takes 32 targets of one child type,
 // a lane each.  Narrow, for launches of few patches (below kWidePatches): a warp

@@ -1092,9 +1092,9 @@ hpfmm_status tree_build(hpfmm_plan *pl, const double *x, const double *y, cudaSt
     set_last_error("tree_build launch: %s", cudaGetErrorString(le));
     return HPFMM_ECUDA;
   }
-  // the reaction tables start on the table stream once the build is done: run during the build, their
-  // FP64-bound blocks slowed its short kernels by a third; after it they
-  // share the SMs with the near field, which leaves the FP64 pipe idle
+  // the reaction tables start on the table stream once the build is done: run
+  // during the build, their FP64-bound blocks slowed its short kernels by a third;
+  // after it they share the SMs with the near field, which leaves the FP64 pipe idle
   if (pl->ev_tree) {
     cudaError_t e = cudaEventRecord(pl->ev_tree, st);
     if (e != cudaSuccess) {
